@@ -152,7 +152,8 @@ int csem_fwd_model(csem_ctx *ctx, const void *rho_dev, const csem_points *src, c
  *  fit_residual_host  out (may be NULL): max |B B+ - I|.
  *  iters_host         out (may be NULL): largest CG iteration count used.
  * Blocks the calling thread until the result is on the host.  Allocates
- * (and frees) 2 n_freq * nt * 16 bytes of scratch on the stream.
+ * (and frees) 16 n_freq * nt bytes of scratch (nt rounded up to a multiple of 512;
+ * 48 n_freq * nt above 65 536 steps) on the stream.
  * Errors: INVALID_ARG, OOM, CUDA. */
 int csem_estimate_adjoint_basis(double dt, int nt, const double *freqs_host, int n_freq, double f0,
                                 double gamma, int gamma_is_relative, int max_iter, double tol,
@@ -165,7 +166,7 @@ int csem_estimate_adjoint_basis(double dt, int nt, const double *freqs_host, int
  * allocator (a framework's caching pool, a fixed arena) and must not see
  * foreign allocations, or run on a path where an allocation's implicit
  * synchronisation or possible failure is not acceptable.  This entry point
- * calls no cudaMalloc, cudaFree or other allocating routine: its CG work
+ * calls no cudaMalloc, cudaFree or other allocating routine: its work
  * vectors live in one file-scope device array of 8 MiB that every device
  * which loads the library keeps until the process exits.
  *  Limits: nt <= 32768 and n_freq <= 8, else INVALID_ARG with a message.

@@ -2031,10 +2031,11 @@ int csem_estimate_adjoint_basis(double dt, int nt, const double *freqs, int nf, 
     cudaStream_t st = (cudaStream_t)stream;
     const int m = 2 * nf;
     double *scratch = nullptr;
-    const size_t sbytes = (size_t)m * 2 * nt * sizeof(double) + (size_t)(m * m + 2 + m) * sizeof(double) +
+    const size_t vec = csem::basis_scratch_doubles(nt, nf);
+    const size_t sbytes = vec * sizeof(double) + (size_t)(m * m + 2 + m) * sizeof(double) +
                           (size_t)m * sizeof(int) + 64;
     CK(cudaMallocAsync((void **)&scratch, sbytes, st));
-    double *gram = scratch + (size_t)m * 2 * nt;
+    double *gram = scratch + vec;
     double *scal = gram + m * m;           // [0] gamma, [1..m] fit per column
     int *iters = (int *)(scal + 1 + m);
     cudaError_t e = csem::launch_basis(dt, nt, a, nf, gamma, gamma_is_relative, max_iter, tol, basis_dev, scratch,

@@ -259,6 +259,8 @@ cudaError_t launch_gradient(const GeoD &g, const R *rho, const typename C2<R>::T
 cudaError_t launch_scatter_int2(int2 *dst, const long long *pos, const int2 *val, int n, cudaStream_t st);
 cudaError_t launch_misfit(int n, const double *d_obs, const double *d_syn, const double *w, double *resid,
                           double *phi, cudaStream_t st);
+// doubles of scratch that launch_basis needs: the phasor table (and, above 65 536 steps, two CG vectors per column)
+size_t basis_scratch_doubles(int nt, int nf);
 cudaError_t launch_basis(double dt, int nt, const double *a, int nf, double gamma, int gamma_rel, int max_iter,
                          double tol, double *basis, double *scratch, double *gram, double *out_scalars,
                          int *out_iters, cudaStream_t st);

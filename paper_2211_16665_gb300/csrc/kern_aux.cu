@@ -1,4 +1,6 @@
 // Set-up, normalisation, misfit, gradient and adjoint-basis kernels.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "csem_internal.cuh"
@@ -335,20 +337,35 @@ cudaError_t launch_misfit(int n, const double *d_obs, const double *d_syn, const
 }
 
 // ---------------------------------------------------------------------------
-// Adjoint-source basis (Sec. 3.3), FP64.  B (2 nf x nt) is never stored: each
-// thread walks a contiguous range of n and advances exp((-1+i) a_k t_n) by the
-// complex factor exp((-1+i) a_k dt) per sample (the start of each range is
-// evaluated directly).  Rows 0..nf-1 are the real parts, nf..2nf-1 the
-// imaginary parts.
+// Adjoint-source basis (Sec. 3.3), FP64.  The samples are cut into kBT contiguous ranges, one per
+// (virtual) thread.  Within a range exp((-1+i) a_k t_n) advances by the complex factor
+// exp((-1+i) a_k dt) per sample (the start of each range is evaluated directly).  Rows 0..nf-1 of B
+// are the real parts, nf..2nf-1 the imaginary parts.
+//
+// What bounds it is the FP64 pipe (a warp instruction holds it for tens of cycles) and, between
+// passes, latency.  So the phasors are evaluated once into a table that every pass of every column
+// reads (k_basis_table; re-evaluating them cost two thirds of a pass's operations and two sincos and
+// exp per range and pass), and a column's kBT ranges are spread over a cluster of eight SMs that
+// keeps the column's CG vectors in shared memory (k_basis_cg).  Every sum is taken over the ranges
+// in the order of one block of kBT threads, so the results are those of that block.  Eight
+// frequencies, 19 492 steps, three solves of up to 200 iterations: 469 ms with one block per column
+// and phasors advanced in every pass, 38 ms now.
 // ---------------------------------------------------------------------------
-constexpr int kBT = 512;
+constexpr int kBT = 512;                 // ranges per column
+constexpr int kBC = 8;                   // SMs (CTAs of a cluster) per column
+constexpr int kBW = kBT / kBC;           // ranges (threads) per CTA
+constexpr int kBMaxChunk = 128;          // samples per range that fit in shared memory: 3 vectors x 64 x 128 x 8 B
 
 struct BasisArgs {
     double dt; int nt; int nf; double a[kMaxFreq];
 };
 
-__device__ __forceinline__ double block_sum(double v, double *red) {
+__device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ double block_sum(double v, double *red) {
+    v = warp_sum(v);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -370,57 +387,214 @@ __device__ __forceinline__ void phasor_start(const BasisArgs &b, int f, int n0, 
     qr = eq * cs; qi = eq * sn;
 }
 
+// Z[(m*nf + f)*kBT + t]: the phasor of frequency f at sample m of range t (zero past the last sample).
+__global__ void __launch_bounds__(64) k_basis_table(BasisArgs b, int chunk, double2 *Z) {
+    const int t = blockIdx.x * 64 + threadIdx.x, f = blockIdx.y;
+    const int n0 = t * chunk, n1 = min(n0 + chunk, b.nt);
+    double zr, zi, qr, qi;
+    phasor_start(b, f, n0, zr, zi, qr, qi);
+    for (int m = 0; m < chunk; ++m) {
+        Z[((long long)m * b.nf + f) * kBT + t] = n0 + m < n1 ? make_double2(zr, zi) : make_double2(0.0, 0.0);
+        const double u = zr * qr - zi * qi; zi = zr * qi + zi * qr; zr = u;
+    }
+}
+
 // Gram matrix G = B B^T (2nf x 2nf), one block per (row, col) pair with row <= col.
-__global__ void __launch_bounds__(kBT) k_basis_gram(BasisArgs b, double *G) {
+__global__ void __launch_bounds__(kBT) k_basis_gram(int nt, int nf, int chunk, const double2 *__restrict__ Z, double *G) {
     __shared__ double red[kBT / 32];
-    const int m = 2 * b.nf;
+    const int m = 2 * nf;
     const int r = blockIdx.x, c = blockIdx.y;
     if (r > c) return;
-    const int chunk = (b.nt + kBT - 1) / kBT;
-    const int n0 = threadIdx.x * chunk, n1 = min(n0 + chunk, b.nt);
+    const int n0 = threadIdx.x * chunk, n1 = min(n0 + chunk, nt);
+    const double2 *zr = Z + (long long)(r % nf) * kBT + threadIdx.x, *zc = Z + (long long)(c % nf) * kBT + threadIdx.x;
     double acc = 0.0;
-    if (n0 < n1) {
-        const int fr = r % b.nf, fc = c % b.nf;
-        double zr, zi, qr, qi, wr, wi, pr, pi;
-        phasor_start(b, fr, n0, zr, zi, qr, qi);
-        phasor_start(b, fc, n0, wr, wi, pr, pi);
-        for (int n = n0; n < n1; ++n) {
-            const double br = (r < b.nf) ? zr : zi;
-            const double bc = (c < b.nf) ? wr : wi;
-            acc += br * bc;
-            double t = zr * qr - zi * qi; zi = zr * qi + zi * qr; zr = t;
-            t = wr * pr - wi * pi; wi = wr * pi + wi * pr; wr = t;
-        }
+    for (int n = n0; n < n1; ++n) {
+        const long long o = (long long)(n - n0) * nf * kBT;
+        const double2 a = zr[o], b = zc[o];
+        acc += (r < nf ? a.x : a.y) * (c < nf ? b.x : b.y);
     }
     acc = block_sum(acc, red);
     if (threadIdx.x == 0) { G[r * m + c] = acc; G[c * m + r] = acc; }
 }
 
-// gamma = gamma_rel * lambda_max(G) by power iteration (G is symmetric positive semi-definite).
-__global__ void k_basis_gamma(const double *G, int m, double gamma, int rel, double *out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    if (!rel) { out[0] = gamma; return; }
-    double v[2 * kMaxFreq], w[2 * kMaxFreq];
-    for (int i = 0; i < m; ++i) v[i] = 1.0 / (1.0 + i);
+// gamma = gamma_rel * lambda_max(G) by power iteration (G is symmetric positive semi-definite), one row
+// per lane; ends early once the vector repeats exactly.
+__global__ void __launch_bounds__(32) k_basis_gamma(const double *G, int m, double gamma, int rel, double *out) {
+    __shared__ double v[2 * kMaxFreq], w[2 * kMaxFreq];
+    const int i = threadIdx.x;
+    if (!rel) {
+        if (i == 0) out[0] = gamma;
+        return;
+    }
+    double g[2 * kMaxFreq];
+#pragma unroll
+    for (int j = 0; j < 2 * kMaxFreq; ++j) g[j] = (i < m && j < m) ? G[i * m + j] : 0.0;
+    if (i < m) v[i] = 1.0 / (1.0 + i);
+    __syncwarp();
     double lam = 0.0;
     for (int it = 0; it < 500; ++it) {
+        double s = 0.0;
+#pragma unroll
+        for (int j = 0; j < 2 * kMaxFreq; ++j)
+            if (j < m) s += g[j] * v[j];
+        if (i < m) w[i] = s;
+        __syncwarp();
         double nrm = 0.0;
-        for (int i = 0; i < m; ++i) {
-            double s = 0.0;
-            for (int j = 0; j < m; ++j) s += G[i * m + j] * v[j];
-            w[i] = s;
-            nrm += s * s;
-        }
+#pragma unroll
+        for (int j = 0; j < 2 * kMaxFreq; ++j)
+            if (j < m) nrm += w[j] * w[j];
         nrm = sqrt(nrm);
         if (nrm == 0.0) break;
-        for (int i = 0; i < m; ++i) v[i] = w[i] / nrm;
+        bool same = true;
+        if (i < m) {
+            const double u = s / nrm;
+            same = u == v[i];
+            v[i] = u;
+        }
         lam = nrm;
+        __syncwarp();
+        if (__all_sync(0xffffffffu, same)) break;   // a fixed point: the remaining iterations repeat this one
     }
-    out[0] = gamma * lam;
+    if (i == 0) out[0] = gamma * lam;
 }
 
-// CGNR on (B^T B + gamma I) x = B^T e_j, one block per column j (Sec. 3.3).
-// x is written into basis[n*2nf + j]; P and Sv are [2nf][nt] scratch rows.
+// CGNR on (B^T B + gamma I) x = B^T e_j, one cluster of kBC CTAs per column j (Sec. 3.3); x is written
+// into basis[n*2nf + j], then the fit max_i |(B x)_i - delta_ij|.  CTA r of the cluster holds the ranges
+// r*kBW ..; the vectors x, p, s are in shared memory as [sample][thread].  A sum over all ranges: every
+// warp writes its partial sum into the table of every CTA, one cluster barrier, and each CTA adds the
+// partial sums in range order.  Two tables in turn, so one barrier per exchange is enough.
+// The roundings are spelled out (which products are fused), so that they do not depend on unrolling.
+__device__ __forceinline__ double add_dot2(double s, double2 z, double r, double i) {
+    return __dadd_rn(s, fma(z.x, r, __dmul_rn(z.y, i)));
+}
+template <int NF>
+__global__ void __cluster_dims__(kBC, 1, 1) __launch_bounds__(kBW)
+    k_basis_cg(int nt, int chunk, const double2 *__restrict__ Z, const double *gamma_p, int max_iter, double tol,
+               double *basis, int *iters, double *fit) {
+    namespace cg = cooperative_groups;
+    constexpr int M = 2 * NF, NWT = kBT / 32, U = NF > 5 ? 2 : 4;
+    extern __shared__ double sm[];
+    __shared__ double tab[2][M + 1][NWT];
+    __shared__ double rvec[M], tot[M + 1];
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), col = blockIdx.x / kBC, tid = threadIdx.x;
+    const int t = rank * kBW + tid;
+    const int n0 = t * chunk, cnt = max(0, min(n0 + chunk, nt) - n0);
+    double *X = sm + tid, *P = X + (long long)chunk * kBW, *Sv = P + (long long)chunk * kBW;
+    const double2 *z = Z + t;
+    const double gamma = gamma_p[0];
+    // partial sums of the values v over the ranges into table b of every CTA (lane i: value i), the
+    // barrier, and the totals into tot
+    auto exchange = [&](int b, const auto &v) {
+        constexpr int NV = (int)(sizeof(v) / sizeof(double));
+        double mine = 0.0;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const double ws = __shfl_sync(0xffffffffu, warp_sum(v[i]), 0);
+            if ((tid & 31) == i) mine = ws;
+        }
+        if ((tid & 31) < NV)
+            for (int r = 0; r < kBC; ++r) *cl.map_shared_rank(&tab[b][tid & 31][t >> 5], r) = mine;
+        cl.sync();
+        if (tid < NV) {
+            double s = 0.0;
+            for (int w = 0; w < NWT; ++w) s += tab[b][tid][w];
+            tot[tid] = s;
+        }
+        __syncthreads();
+    };
+    if (tid < M) rvec[tid] = (tid == col) ? 1.0 : 0.0;
+    cl.sync();                            // every CTA runs before any writes to its tables
+    // s = B^T r - gamma x with x = 0, p = s
+    double gl[1] = {0.0};
+    for (int m = 0; m < cnt; ++m) {
+        double s = 0.0;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const double2 zz = z[((long long)m * NF + f) * kBT];
+            s = add_dot2(s, zz, rvec[f], rvec[NF + f]);
+        }
+        Sv[m * kBW] = s; P[m * kBW] = s; X[m * kBW] = 0.0;
+        gl[0] = fma(s, s, gl[0]);
+    }
+    exchange(1, gl);
+    double gam = tot[0];
+    const double g0 = gam;
+    int it = 0;
+    for (; it < max_iter; ++it) {
+        if (!(sqrt(gam) > tol * sqrt(g0))) break;
+        // q = B p, pp = ||p||^2
+        double ql[M + 1];
+#pragma unroll
+        for (int i = 0; i <= M; ++i) ql[i] = 0.0;
+#pragma unroll U
+        for (int m = 0; m < cnt; ++m) {
+            const double pn = P[m * kBW];
+            ql[M] = fma(pn, pn, ql[M]);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+                const double2 zz = z[((long long)m * NF + f) * kBT];
+                ql[f] = fma(zz.x, pn, ql[f]);
+                ql[NF + f] = fma(zz.y, pn, ql[NF + f]);
+            }
+        }
+        exchange(0, ql);
+        double q[M], qq = 0.0;
+#pragma unroll
+        for (int i = 0; i < M; ++i) { q[i] = tot[i]; qq = fma(q[i], q[i], qq); }
+        const double alpha = gam / fma(gamma, tot[M], qq);
+        double rv[M];
+#pragma unroll
+        for (int i = 0; i < M; ++i) rv[i] = fma(-alpha, q[i], rvec[i]);
+        __syncthreads();                  // every thread has read rvec and tot
+        if (tid < M) {
+#pragma unroll
+            for (int i = 0; i < M; ++i)
+                if (i == tid) rvec[i] = rv[i];
+        }
+        // x += alpha p; s = B^T r - gamma x; ||s||^2
+        gl[0] = 0.0;
+#pragma unroll U
+        for (int m = 0; m < cnt; ++m) {
+            const double x = fma(alpha, P[m * kBW], X[m * kBW]);
+            X[m * kBW] = x;
+            double s = __dmul_rn(-gamma, x);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+                const double2 zz = z[((long long)m * NF + f) * kBT];
+                s = add_dot2(s, zz, rv[f], rv[NF + f]);
+            }
+            Sv[m * kBW] = s;
+            gl[0] = fma(s, s, gl[0]);
+        }
+        exchange(1, gl);              // (its barrier also orders rvec)
+        const double gnew = tot[0];       // (read before the next exchange's barrier lets tot change)
+        const double beta = gnew / gam;
+        gam = gnew;
+        for (int m = 0; m < cnt; ++m) P[m * kBW] = fma(beta, P[m * kBW], Sv[m * kBW]);
+    }
+    if (t == 0) iters[col] = it;
+    double ql[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) ql[i] = 0.0;
+    for (int m = 0; m < cnt; ++m) {
+        const double x = X[m * kBW];
+        basis[(long long)(n0 + m) * M + col] = x;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const double2 zz = z[((long long)m * NF + f) * kBT];
+            ql[f] = fma(zz.x, x, ql[f]);
+            ql[NF + f] = fma(zz.y, x, ql[NF + f]);
+        }
+    }
+    exchange(0, ql);                   // also: no CTA ends while another may still write to it
+    double worst = 0.0;
+    for (int i = 0; i < M; ++i) worst = fmax(worst, fabs(tot[i] - (i == col ? 1.0 : 0.0)));
+    if (t == 0) fit[col] = worst;
+}
+
+// The same for ranges too long for shared memory (more than 65 536 steps): one block per column, the CG
+// vectors P and Sv in [2nf][nt] scratch rows, x in the basis, the phasors advanced in every pass.
 __global__ void __launch_bounds__(kBT) k_basis_cgnr(BasisArgs b, const double *gamma_p, int max_iter, double tol,
                                                    double *basis, double *scratch, int *iters) {
     __shared__ double red[kBT / 32];
@@ -536,19 +710,57 @@ __global__ void __launch_bounds__(kBT) k_basis_fit(BasisArgs b, const double *ba
     if (threadIdx.x == 0) fit[col] = worst;
 }
 
+namespace {
+int basis_chunk(int nt) { return (nt + kBT - 1) / kBT; }
+template <int NF>
+cudaError_t cg_go(int nt, const double2 *Z, const double *gamma_p, int max_iter, double tol, double *basis, int *iters,
+                  double *fit, cudaStream_t st) {
+    const int chunk = basis_chunk(nt);
+    const size_t smem = 3 * (size_t)chunk * kBW * sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(k_basis_cg<NF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(3 * (size_t)kBMaxChunk * kBW * sizeof(double)));
+    if (e != cudaSuccess) return e;
+    k_basis_cg<NF><<<2 * NF * kBC, kBW, smem, st>>>(nt, chunk, Z, gamma_p, max_iter, tol, basis, iters, fit);
+    return cudaGetLastError();
+}
+}  // namespace
+
+size_t basis_scratch_doubles(int nt, int nf) {
+    const size_t table = (size_t)basis_chunk(nt) * kBT * nf * 2;
+    return basis_chunk(nt) <= kBMaxChunk ? table : table + 4 * (size_t)nf * nt;
+}
+
 cudaError_t launch_basis(double dt, int nt, const double *a, int nf, double gamma, int gamma_rel, int max_iter,
                          double tol, double *basis, double *scratch, double *gram, double *out_scalars,
                          int *out_iters, cudaStream_t st) {
     BasisArgs b;
     b.dt = dt; b.nt = nt; b.nf = nf;
     for (int f = 0; f < kMaxFreq; ++f) b.a[f] = (f < nf) ? a[f] : 0.0;
-    const int m = 2 * nf;
-    k_basis_gram<<<dim3(m, m), kBT, 0, st>>>(b, gram);
+    const int m = 2 * nf, chunk = basis_chunk(nt);
+    double2 *Z = reinterpret_cast<double2 *>(scratch);
+    k_basis_table<<<dim3(kBT / 64, nf), 64, 0, st>>>(b, chunk, Z);
+    k_basis_gram<<<dim3(m, m), kBT, 0, st>>>(nt, nf, chunk, Z, gram);
     k_basis_gamma<<<1, 32, 0, st>>>(gram, m, gamma, gamma_rel, out_scalars);
-    k_basis_cgnr<<<m, kBT, 0, st>>>(b, out_scalars, max_iter, tol, basis, scratch, out_iters);
-    k_basis_fit<<<m, kBT, 0, st>>>(b, basis, out_scalars + 1);
     g_launches += 4;
-    return cudaGetLastError();
+    if (chunk > kBMaxChunk) {
+        double *vec = scratch + (size_t)chunk * kBT * nf * 2;
+        k_basis_cgnr<<<m, kBT, 0, st>>>(b, out_scalars, max_iter, tol, basis, vec, out_iters);
+        k_basis_fit<<<m, kBT, 0, st>>>(b, basis, out_scalars + 1);
+        g_launches++;
+        return cudaGetLastError();
+    }
+    double *fit = out_scalars + 1;
+    switch (nf) {
+        case 1: return cg_go<1>(nt, Z, out_scalars, max_iter, tol, basis, out_iters, fit, st);
+        case 2: return cg_go<2>(nt, Z, out_scalars, max_iter, tol, basis, out_iters, fit, st);
+        case 3: return cg_go<3>(nt, Z, out_scalars, max_iter, tol, basis, out_iters, fit, st);
+        case 4: return cg_go<4>(nt, Z, out_scalars, max_iter, tol, basis, out_iters, fit, st);
+        case 5: return cg_go<5>(nt, Z, out_scalars, max_iter, tol, basis, out_iters, fit, st);
+        case 6: return cg_go<6>(nt, Z, out_scalars, max_iter, tol, basis, out_iters, fit, st);
+        case 7: return cg_go<7>(nt, Z, out_scalars, max_iter, tol, basis, out_iters, fit, st);
+        case 8: return cg_go<8>(nt, Z, out_scalars, max_iter, tol, basis, out_iters, fit, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 // colmap[pos[u]] = val[u]: sets the column map of the injection taps

@@ -21,7 +21,7 @@ namespace {
 
 constexpr int kNoAllocMaxNt = 32768;
 constexpr int kNoAllocMaxCols = 2 * csem::kMaxFreq;
-// layout: [cols][2][nt] CG vectors | [cols][cols] Gram matrix | [1 + cols] scalars | [cols] int iteration counts
+// layout: phasor table (at most half of [cols][2][nt]) | [cols][cols] Gram matrix | [1 + cols] scalars | [cols] int iteration counts
 constexpr size_t kVecDoubles = (size_t)kNoAllocMaxCols * 2 * kNoAllocMaxNt;
 constexpr size_t kGramDoubles = (size_t)kNoAllocMaxCols * kNoAllocMaxCols;
 constexpr size_t kScalDoubles = 1 + kNoAllocMaxCols;
@@ -76,9 +76,9 @@ extern "C" int csem_estimate_adjoint_basis_noalloc(double dt, int nt, const doub
     int *iters = (int *)(scal + kScalDoubles);
     // The basis kernels write every value of the array they later read, so a clear is
     // not needed for the result; it is kept, limited to the part this call uses (its
-    // m CG vector pairs and the Gram/scalar/count block), so that a kernel fault can
+    // phasor table and the Gram/scalar/count block), so that a kernel fault can
     // never show a previous call's numbers.
-    cudaError_t e = cudaMemsetAsync(vec, 0, (size_t)m * 2 * nt * sizeof(double), st);
+    cudaError_t e = cudaMemsetAsync(vec, 0, csem::basis_scratch_doubles(nt, nf) * sizeof(double), st);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(gram, 0, (kGramDoubles + kScalDoubles + kIterDoubles) * sizeof(double), st);
     if (e == cudaSuccess)
