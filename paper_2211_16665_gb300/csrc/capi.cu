@@ -713,11 +713,16 @@ template <typename R>
 int coef_init(csem_ctx *c, const void *rho, cudaStream_t st) {
     const long long cells = (long long)c->nx * c->ny * c->nz;
     const R *rho_h = (const R *)rho, *rho_z = rho_h + (c->vti ? cells : 0);
-    CK(csem::launch_coef_init<R>(geo(c), rho_h, rho_z, (R *)c->d_cE, 2.0 * c->w0 * c->dt, c->d_bad, st));
+    bool masked = false;
+    R *cEm = nullptr;
+    if constexpr (sizeof(R) == 4) cEm = c->d_cEm;
+    CK(csem::launch_coef_init<R>(geo(c), rho_h, rho_z, (R *)c->d_cE, cEm, &masked, 2.0 * c->w0 * c->dt, c->d_bad, st));
     if constexpr (sizeof(R) == 4) {
-        if (c->d_cEm) CK(csem::launch_mask_coef(step_params<float>(c, false, nullptr), (const float *)c->d_cE, c->d_cEm, st));
-        if (c->d_q) CK(csem::launch_qcell(geo(c), (const float *)rho_h, (const float *)rho_z, c->d_q,
-                                          c->vti ? c->d_q + c->vol : nullptr, st));
+        if (c->d_cEm && !masked)
+            CK(csem::launch_mask_coef(step_params<float>(c, false, nullptr), (const float *)c->d_cE, c->d_cEm, st));
+        if (c->d_q && c->FZ_by && !c->FZ_ws)     // only the one-pass step reads V sigma
+            CK(csem::launch_qcell(geo(c), (const float *)rho_h, (const float *)rho_z, c->d_q,
+                                  c->vti ? c->d_q + c->vol : nullptr, st));
     }
     return CSEM_OK;
 }

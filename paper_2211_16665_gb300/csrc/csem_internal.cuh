@@ -242,10 +242,11 @@ struct GeoD {                      // double-precision geometry for set-up and g
 };
 // q = V sigma per cell on the lattice (sigma_h into qh; sigma_v into qv when qv is not NULL)
 cudaError_t launch_qcell(const GeoD &g, const float *rho, const float *rho_z, float *qh, float *qv, cudaStream_t st);
+// dt/eps on every edge from the cell resistivity (rho_z on the z edges: rho_v of a VTI medium, else rho);
+// cEm (FP32, may be NULL): also its copy with the PEC edges zeroed, *masked tells whether it was written
 template <typename R>
-// dt/eps on every edge from the cell resistivity (rho_z on the z edges: rho_v of a VTI medium, else rho)
-cudaError_t launch_coef_init(const GeoD &g, const R *rho, const R *rho_z, R *cE, double two_w0_dt, int *bad_flag,
-                             cudaStream_t st);
+cudaError_t launch_coef_init(const GeoD &g, const R *rho, const R *rho_z, R *cE, R *cEm, bool *masked,
+                             double two_w0_dt, int *bad_flag, cudaStream_t st);
 template <typename R>
 cudaError_t launch_finalize_volume(typename C2<R>::T *acc, const typename C2<R>::T *comp, long long vol, int S,
                                    int nf, const double2 *alpha, cudaStream_t st);
