@@ -300,7 +300,9 @@ __device__ __forceinline__ void dft_receivers(const StepParams<R> &p, const Poin
 
 // Transform of the snapshots n0 .. n0+cnt-1 (n0 = *step + n0_off).
 // The first blocks take the receivers (they start first), the others
-// the volume entries (block -> (vb, c, s)).  CNT > 0:
+// the volume entries (block -> (vb, c, s)).  The first flush of a run (n0 = 0) starts
+// from zero accumulators without reading them, in this and the bulk-copy kernels, so a run
+// does not clear its volumes.  CNT > 0:
 // cnt is a multiple of CNT and the snapshots are read in unrolled groups of
 // CNT; CNT = 0: any cnt, one snapshot at a time.
 template <typename R, bool VOL, bool KAHAN, int CNT>
@@ -335,8 +337,11 @@ __global__ void __launch_bounds__(kBlock) k_dft(const StepParams<R> p, const Poi
 #pragma unroll
     for (int f = 0; f < kMaxFreq; ++f)
         if (f < p.nf) {
-            acc[f] = A[(long long)f * p.vol];
-            if (KAHAN) cmp[f] = C[(long long)f * p.vol];
+            acc[f].x = acc[f].y = cmp[f].x = cmp[f].y = R(0);
+            if (n0 > 0) {
+                acc[f] = A[(long long)f * p.vol];
+                if (KAHAN) cmp[f] = C[(long long)f * p.vol];
+            }
         }
     // block sum of the products with plain FMAs, then one compensated addition
     // of the block sum to the running accumulator
@@ -489,13 +494,13 @@ __global__ void __launch_bounds__(kBulkThreads, bulk_minb<MS>()) k_dft_bulk(cons
     __syncthreads();
     if (threadIdx.x == 0) {
         const uint32_t rb = (uint32_t)rows * sizeof(float), cb = (uint32_t)rows * sizeof(float2);
-        mbar_expect_tx(&bar, MS * rb + p.nf * cb * (KAHAN ? 2u : 1u) + (uint32_t)p.fault_tx);
+        mbar_expect_tx(&bar, MS * rb + (n0 > 0 ? p.nf * cb * (KAHAN ? 2u : 1u) : 0u) + (uint32_t)p.fault_tx);
         int sl = n0 % p.nslot;
         for (int m = 0; m < MS; ++m) {
             bulk_g2s(ring_s + m * kBlock, ring + (long long)sl * 3 * p.vol, rb, &bar);
             sl = (sl + 1 == p.nslot) ? 0 : sl + 1;
         }
-        for (int f = 0; f < p.nf; ++f) {
+        for (int f = 0; f < p.nf && n0 > 0; ++f) {
             bulk_g2s(acc_s + f * kBlock, A + (long long)f * p.vol, cb, &bar);
             if (KAHAN) bulk_g2s(cmp_s + f * kBlock, C + (long long)f * p.vol, cb, &bar);
         }
@@ -538,9 +543,10 @@ __global__ void __launch_bounds__(kBulkThreads, bulk_minb<MS>()) k_dft_bulk(cons
     for (int f = 0; f < NF; ++f) {
         if (f >= p.nf) break;
         const float2 s0 = unpack_f32x2(p0[f]), s1 = unpack_f32x2(p1[f]);
-        float4 a = *reinterpret_cast<const float4 *>(acc_s + f * kBlock + t2);   // entries t2, t2+1
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 a = n0 > 0 ? *reinterpret_cast<const float4 *>(acc_s + f * kBlock + t2) : z;   // entries t2, t2+1
         if (KAHAN) {
-            float4 cc = *reinterpret_cast<const float4 *>(cmp_s + f * kBlock + t2);
+            float4 cc = n0 > 0 ? *reinterpret_cast<const float4 *>(cmp_s + f * kBlock + t2) : z;
             kahan_add(a.x, cc.x, s0.x);
             kahan_add(a.y, cc.y, s0.y);
             kahan_add(a.z, cc.z, s1.x);
@@ -628,7 +634,7 @@ __global__ void __launch_bounds__(kBulkThreads, stream_minb(NF)) k_dft_stream(co
     };
     if (threadIdx.x == 0) {
         for (int ch = 0; ch < kStN; ++ch) issue(ch);
-        if (SACC) {
+        if (SACC && n0 > 0) {
             mbar_expect_tx(&abar, p.nf * cb * (KAHAN ? 2u : 1u));
             for (int f = 0; f < p.nf; ++f) {
                 bulk_g2s(acc_s + f * kBlock, A + (long long)f * p.vol, cb, &abar);
@@ -672,14 +678,14 @@ __global__ void __launch_bounds__(kBulkThreads, stream_minb(NF)) k_dft_stream(co
         }
     }
     const bool done = (ch == NCH);
-    if (SACC && done && ok) ok = mbar_wait_bounded(&abar, 0);
+    if (SACC && n0 > 0 && done && ok) ok = mbar_wait_bounded(&abar, 0);
     if (__syncthreads_or(!ok)) {
         if (threadIdx.x == 0) {
             atomicOr(err, kErrFlushWait);
             // copies issued and not consumed: chunks ch .. issued - 1 (each in its own stage), and
             // the accumulators; a wait that already completed returns at once
             for (int x = ch; x < issued; ++x) mbar_wait_bounded(&full[x & (kStN - 1)], (uint32_t)(x / kStN) & 1u);
-            if (SACC) mbar_wait_bounded(&abar, 0);
+            if (SACC && n0 > 0) mbar_wait_bounded(&abar, 0);
         }
         return;
     }
@@ -689,11 +695,15 @@ __global__ void __launch_bounds__(kBulkThreads, stream_minb(NF)) k_dft_stream(co
         if (f >= p.nf) break;
         const float2 s0 = unpack_f32x2(p0[f]), s1 = unpack_f32x2(p1[f]);
         // entries t2, t2+1
-        float4 a = SACC ? *reinterpret_cast<const float4 *>(acc_s + f * kBlock + t2)
-                        : *reinterpret_cast<const float4 *>(A + (long long)f * p.vol + t2);
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), cc = a;
+        if (n0 > 0) {
+            a = SACC ? *reinterpret_cast<const float4 *>(acc_s + f * kBlock + t2)
+                     : *reinterpret_cast<const float4 *>(A + (long long)f * p.vol + t2);
+            if (KAHAN)
+                cc = SACC ? *reinterpret_cast<const float4 *>(cmp_s + f * kBlock + t2)
+                          : *reinterpret_cast<const float4 *>(C + (long long)f * p.vol + t2);
+        }
         if (KAHAN) {
-            float4 cc = SACC ? *reinterpret_cast<const float4 *>(cmp_s + f * kBlock + t2)
-                             : *reinterpret_cast<const float4 *>(C + (long long)f * p.vol + t2);
             kahan_add(a.x, cc.x, s0.x);
             kahan_add(a.y, cc.y, s0.y);
             kahan_add(a.z, cc.z, s1.x);
