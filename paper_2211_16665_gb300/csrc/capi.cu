@@ -1687,19 +1687,16 @@ int csem_create(csem_ctx **out, const csem_grid *g, const csem_opts *o) {
                 rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
         }
     }
-    // FP32, nx even: tap increments and padded tables (and for the fourth order the masked
-    // dt/eps of its lean kernels); second order also the fused one-pass step's per-cell
-    // material and widths, and for the lean split kernels (nx a multiple of 4) the CPML
-    // memory in 12 volume arrays per source, kept when it fits
-    if (rc == CSEM_OK && c->precision == 32 && c->nx % 2 == 0) {
+    // FP32: tap increments, padded tables and the masked dt/eps of the lean kernels (fourth order: nx even);
+    // second order also the CPML memory of the lean split kernels in 12 volume arrays per source, kept when it
+    // fits, and, nx even, the fused one-pass step's per-cell material and widths
+    if (rc == CSEM_OK && c->precision == 32 && (c->order == 2 || c->nx % 2 == 0)) {
         step(dalloc(c, &c->d_inc, (size_t)kChunk * S * std::max(8, NR * 8) * sizeof(float)));
         step(dalloc(c, &c->d_tapk, (size_t)std::max(S, NR) * 8 * sizeof(int)));
         step(upload_lean_tables(c));
-        if (c->order == 4) {                 // lean fourth-order kernels: masked dt/eps
-            step(dalloc(c, &c->d_cEm, 3 * (size_t)c->vol * sizeof(float)));
-            if (rc == CSEM_OK && cudaMemset(c->d_cEm, 0, 3 * (size_t)c->vol * sizeof(float)) != cudaSuccess)
-                rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
-        }
+        step(dalloc(c, &c->d_cEm, 3 * (size_t)c->vol * sizeof(float)));
+        if (rc == CSEM_OK && cudaMemset(c->d_cEm, 0, 3 * (size_t)c->vol * sizeof(float)) != cudaSuccess)
+            rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
     }
     if (rc == CSEM_OK && c->order == 2 && c->precision == 32 && c->nx % 2 == 0) {
         if (rc == CSEM_OK) step(upload_geo_tables(c));
@@ -1709,15 +1706,15 @@ int csem_create(csem_ctx **out, const csem_grid *g, const csem_opts *o) {
         // autotuner times the fused step on finite arithmetic
         if (rc == CSEM_OK && cudaMemset(c->d_q, 0x3f, qb) != cudaSuccess)
             rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
+    }
+    if (rc == CSEM_OK && c->order == 2 && c->precision == 32) {
         size_t free_b = 0, total_b = 0;
         cudaMemGetInfo(&free_b, &total_b);
-        const double need = ((double)S * 12 + 3) * c->vol * sizeof(float);
-        if (rc == CSEM_OK && c->nx % 4 == 0 && need < 0.25 * (double)free_b) {
+        const double need = (double)S * 12 * c->vol * sizeof(float);
+        if (need < 0.25 * (double)free_b) {
             step(dalloc(c, &c->d_psiL, (size_t)S * 12 * c->vol * sizeof(float)));
-            step(dalloc(c, &c->d_cEm, 3 * (size_t)c->vol * sizeof(float)));
-            step(dalloc(c, &c->d_wave, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)));
-            if (rc == CSEM_OK && (cudaMemset(c->d_cEm, 0, 3 * (size_t)c->vol * sizeof(float)) != cudaSuccess ||
-                                  cudaMemset(c->d_wave, 0, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)) != cudaSuccess))
+            if (c->nx % 4 == 0) step(dalloc(c, &c->d_wave, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)));
+            if (rc == CSEM_OK && c->d_wave && cudaMemset(c->d_wave, 0, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)) != cudaSuccess)
                 rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
         }
     }
@@ -1971,7 +1968,7 @@ int csem_set_launch(csem_ctx *c, const int *cfg) {
             return l == 0 || ((l == 1 || l == 2) && (kz == 1 || kz == 2 || kz == 4) &&
                               (mb == 6 || mb == 8 || (mb == 4 && l == 2)));
         };
-        if (!c->d_psiL || !ok(lh, kzh, mbh) || !ok(le, kze, mbe))
+        if (!c->d_psiL || c->nx % 4 != 0 || !ok(lh, kzh, mbh) || !ok(le, kze, mbe))
             return fail(CSEM_ERR_INVALID_ARG, "lean kernels: FP32, nx a multiple of 4, 1 or 2 cells, 1/2/4 planes, 6 or 8 (2 cells: 4, 6 or 8) blocks/SM");
     }
     if (th || te) {

@@ -1,13 +1,14 @@
 // Lean FP32 H and E step kernels (Sec. 2, Eq. 4 with the unsplit CPML): W
 // consecutive cells (W = 1 or 2; i a multiple of W) of one (j, k) row per
-// thread, the cell range [0,nx) x [0,ny) x [0,nz) (nx a multiple of 4), KZ
-// planes along z per thread.  They compute what the scalar kernels compute,
+// thread, the cell range [0,nx) x [0,ny) x [0,nz), KZ planes along z per thread.
+// With nx odd the last thread's second cell is the row's entry nx: its dt/eps and
+// spacings are zero, so its values stay zero.  They compute what the scalar kernels compute,
 // entry by entry, with every load of a plane independent of the others, so that
 // a plane's loads are in flight together:
 //  * the CPML memory lives in arrays of its own (12 per source: 0-5 for H, 6-11
 //    for E).  The y- and z-slab arrays have the field layout.  The x-slab arrays
-//    (3, 4, 9, 10) are compact: row (k, j) holds the 2*nxs cells i < nxs and
-//    i >= nx - nxs (nxs = npml rounded up to even), so the slab entries of
+//    (3, 4, 9, 10) are compact: row (k, j) holds the cells i < lo and i >= hi (lo =
+//    npml rounded up, hi = nx - npml rounded down to even), so the slab entries of
 //    consecutive rows are contiguous;
 //  * the coefficient tables are padded to whole 16-byte groups, and the CPML
 //    coefficients are zero off the slabs and on the outer nodes.  A cell in the
@@ -113,7 +114,7 @@ template <int W> __device__ __forceinline__ Vec<W> up(const Vec<W> &a, float nex
 
 // Per-thread constants shared by the planes of a lean kernel.
 template <int W> struct LeanRow {
-    int i, j, nxs, ixs;
+    int i, j, nxs, ixs;                  // nxs: slab entries per row, ixs: the cells' place among them
     bool xs, ys;
     Vec<W> ihx, bx, ax;
     float ihy, by, ay;
@@ -123,9 +124,10 @@ __device__ __forceinline__ void lean_row(const StepParams<float> &p, const AxisT
                                          bool half, int i, int j, LeanRow<W> &r) {
     const int npml = p.npml;
     r.i = i; r.j = j;
-    r.nxs = (npml + 1) & ~1;
-    r.xs = (i < r.nxs) || (i + W > p.nx - r.nxs);
-    r.ixs = (i < r.nxs) ? i : i - (p.nx - 2 * r.nxs);
+    const int lo = (npml + 1) & ~1, hi = (p.nx - npml) & ~1;
+    r.nxs = lo + ((p.nx + 1) & ~1) - hi;
+    r.xs = npml > 0 && (i < lo || i >= hi);
+    r.ixs = (i < lo) ? i : i - hi + lo;
     r.ihx = ldc<W>((half ? tx.ih_h : tx.ih_n) + i);
     r.bx = ldc<W>((half ? tx.b_h : tx.b_n) + i);
     r.ax = ldc<W>((half ? tx.a_h : tx.a_n) + i);
@@ -167,7 +169,7 @@ __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float 
     const float eyn = __ldg(E + vol + idx + W), ezn = __ldg(E + 2 * vol + idx + W);
     const float ihz = __ldg(p.lz.ih_h + k);
     Vec<W> hx = ldw<W>(H + idx), hy = ldw<W>(H + vol + idx), hz = ldw<W>(H + 2 * vol + idx);
-    const int xo = (k * p.ny + r.j) * (2 * r.nxs) + r.ixs;
+    const int xo = (k * p.ny + r.j) * r.nxs + r.ixs;
     float *px3 = ps + 3 * vol + xo, *px4 = ps + 4 * vol + xo;
     Vec<W> q3 = ldw<W>(r.xs ? px3 : p.lzero), q4 = ldw<W>(r.xs ? px4 : p.lzero);
     bool zs = false, ys = false;
@@ -295,7 +297,7 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
     const Vec<W> eo0 = ldc<W>(Eo + idx), eo1 = ldc<W>(Eo + vol + idx), eo2 = ldc<W>(Eo + 2 * vol + idx);
     const Vec<W> c0 = ldc<W>(cE + idx), c1 = ldc<W>(cE + vol + idx), c2 = ldc<W>(cE + 2 * vol + idx);
     const float ihz = __ldg(p.lz.ih_n + k);
-    const int xo = (k * p.ny + r.j) * (2 * r.nxs) + r.ixs;
+    const int xo = (k * p.ny + r.j) * r.nxs + r.ixs;
     float *px3 = ps + 3 * vol + xo, *px4 = ps + 4 * vol + xo;
     Vec<W> q3 = ldw<W>(r.xs ? px3 : p.lzero), q4 = ldw<W>(r.xs ? px4 : p.lzero);
     bool zs = false, ys = false;
@@ -560,7 +562,7 @@ namespace {
 template <int W, int KZ, int MB>
 void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h) {
     const dim3 block(kLeanX, kLeanRows);
-    const int nv = p.nx / W;
+    const int nv = (p.nx + W - 1) / W;
     const dim3 grid((nv + kLeanX - 1) / kLeanX, (p.ny + kLeanRows - 1) / kLeanRows, ((p.nz + KZ - 1) / KZ) * S);
     if (h) k_h_lean<W, KZ, MB><<<grid, block, 0, st>>>(p, jstep);
     else k_e_lean<W, KZ, MB><<<grid, block, 0, st>>>(p, jstep);
@@ -578,7 +580,7 @@ bool lean_kz(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool
 
 cudaError_t launch_field_lean(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int w, int kz,
                               int mb) {
-    if (p.nx % 4 != 0 || !p.psiL || !p.cEm || !p.lx.ih_n || !p.lzero) return cudaErrorInvalidValue;
+    if (!p.psiL || !p.cEm || !p.lx.ih_n || !p.lzero) return cudaErrorInvalidValue;
     bool ok = false;
     if (w == 1 && mb == 6) ok = lean_kz<1, 6>(p, S, jstep, st, h, kz);
     else if (w == 1 && mb == 8) ok = lean_kz<1, 8>(p, S, jstep, st, h, kz);
