@@ -27,11 +27,11 @@ __device__ __forceinline__ R d_half(const R *__restrict__ F, long long at, long 
 
 // d/da at the node pos (of n) of a half-node-located field F, F[at] at half node pos
 template <typename R>
-__device__ __forceinline__ R d_node(const R *__restrict__ F, long long at, long long s, int pos, int n,
+__device__ __forceinline__ R d_node(const R *F, long long at, long long s, int pos, int n,
                                     const R *__restrict__ w) {
     const R *wr = w + 4 * pos;
-    R d = ld(wr + 1) * ld(F + at - s) + ld(wr + 2) * ld(F + at);
-    if (pos >= 2 && pos <= n - 2) d = ld(wr) * ld(F + at - 2 * s) + d + ld(wr + 3) * ld(F + at + s);
+    R d = ld(wr + 1) * F[at - s] + ld(wr + 2) * F[at];
+    if (pos >= 2 && pos <= n - 2) d = ld(wr) * F[at - 2 * s] + d + ld(wr + 3) * F[at + s];
     return d;
 }
 
@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(kHoX *kHoY) k_h_ho(const StepParams<R> p, cons
     const int nzb = (p.NZ + kHoZ - 1) / kHoZ;
     const int s = blockIdx.z / nzb, k0 = (blockIdx.z % nzb) * kHoZ;
     if (i >= p.NX || j >= p.NY) return;
+    pdl_wait();
     const int n = *p.step + jstep;
     const long long vol = p.vol, plane = p.plane, pitch = p.pitch;
     const R *__restrict__ Ex = p.ering + (long long)s * p.ering_stride + (long long)(n % p.nslot) * 3 * vol;
@@ -94,6 +95,7 @@ __global__ void __launch_bounds__(kHoX *kHoY) k_e_ho(const StepParams<R> p, cons
     const int nzb = (p.NZ + kHoZ - 1) / kHoZ;
     const int s = blockIdx.z / nzb, k0 = (blockIdx.z % nzb) * kHoZ;
     if (i >= p.NX || j >= p.NY) return;
+    pdl_wait();
     const int n = *p.step + jstep;
     const long long vol = p.vol, plane = p.plane, pitch = p.pitch;
     const R *__restrict__ Eo = p.ering + (long long)s * p.ering_stride + (long long)(n % p.nslot) * 3 * vol;
@@ -208,6 +210,7 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
     const int s = blockIdx.z % S, k0 = (blockIdx.z / S) * KZ;
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
+    pdl_wait();
     const int n = *p.step + jstep;
     const int nx = p.nx, ny = p.ny, nz = p.nz, npml = p.npml;
     const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch;
@@ -280,6 +283,7 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
     const int s = blockIdx.z % S, k0 = (blockIdx.z / S) * KZ;
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
+    pdl_wait();
     const int n = *p.step + jstep;
     const int nx = p.nx, ny = p.ny, nz = p.nz, npml = p.npml;
     const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch;
@@ -304,22 +308,22 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
     // z window of Hx, Hy at the thread's cells: planes k-2, k-1, k (k+1 loaded per step)
     const int base = j * pitch + i;
     const int ka = (k0 >= 2) ? k0 - 2 : 0, kb = (k0 >= 1) ? k0 - 1 : 0;
-    float2 xa = f2g(Hx + ka * plane + base), xb = f2g(Hx + kb * plane + base), xc = f2g(Hx + k0 * plane + base);
-    float2 ya = f2g(Hy + ka * plane + base), yb = f2g(Hy + kb * plane + base), yc = f2g(Hy + k0 * plane + base);
+    float2 xa = f2w(Hx + ka * plane + base), xb = f2w(Hx + kb * plane + base), xc = f2w(Hx + k0 * plane + base);
+    float2 ya = f2w(Hy + ka * plane + base), yb = f2w(Hy + kb * plane + base), yc = f2w(Hy + k0 * plane + base);
 #pragma unroll
     for (int kk = 0; kk < KZ; ++kk) {
         const int k = k0 + kk;
         if (k >= k1) break;
         const int idx = k * plane + base;
-        const float2 xd = f2g(Hx + idx + plane), yd = f2g(Hy + idx + plane);   // plane k+1 <= nz
+        const float2 xd = f2w(Hx + idx + plane), yd = f2w(Hy + idx + plane);   // plane k+1 <= nz
         const float4 wz = f4g(w.wzn + 4 * k);
         // x neighbours of Hy, Hz (plane k): values at i-2 .. i+2
-        const float2 hym = f2g(Hy + idx + im2), hzm = f2g(Hz + idx + im2);
-        const float2 hz01 = f2g(Hz + idx);
-        const float hy2 = __ldg(Hy + idx + 2), hz2 = __ldg(Hz + idx + 2);
+        const float2 hym = f2w(Hy + idx + im2), hzm = f2w(Hz + idx + im2);
+        const float2 hz01 = f2w(Hz + idx);
+        const float hy2 = Hy[idx + 2], hz2 = Hz[idx + 2];
         // y neighbours of Hx, Hz (plane k): rows j-2, j-1, j+1
-        const float2 hxm2 = f2g(Hx + idx + jm2), hxm1 = f2g(Hx + idx + jm1), hxp1 = f2g(Hx + idx + pitch);
-        const float2 hzm2 = f2g(Hz + idx + jm2), hzm1 = f2g(Hz + idx + jm1), hzp1 = f2g(Hz + idx + pitch);
+        const float2 hxm2 = f2w(Hx + idx + jm2), hxm1 = f2w(Hx + idx + jm1), hxp1 = f2w(Hx + idx + pitch);
+        const float2 hzm2 = f2w(Hz + idx + jm2), hzm1 = f2w(Hz + idx + jm1), hzp1 = f2w(Hz + idx + pitch);
         const float2 e0 = f2g(Eo + idx), e1 = f2g(Eo + vol + idx), e2 = f2g(Eo + 2 * vol + idx);
         const float2 c0 = f2g(cE + idx), c1 = f2g(cE + vol + idx), c2 = f2g(cE + 2 * vol + idx);
         float2 dHz_dy = dot4(wy, hzm2, hzm1, hz01, hzp1), dHy_dz = dot4(wz, ya, yb, yc, yd);
@@ -359,8 +363,8 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
 template <int KZ, int MB>
 void go_ho4k(const StepParams<float> &p, const HoTab<float> &w, int S, int jstep, cudaStream_t st, bool h) {
     const dim3 grid((unsigned)((p.nx / 2 + 31) / 32), (unsigned)((p.ny + 3) / 4), (unsigned)(((p.nz + KZ - 1) / KZ) * S));
-    if (h) k_h_ho4<KZ, MB><<<grid, dim3(32, 4), 0, st>>>(p, w, jstep);
-    else k_e_ho4<KZ, MB><<<grid, dim3(32, 4), 0, st>>>(p, w, jstep);
+    if (h) launch_pdl(k_h_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep);
+    else launch_pdl(k_e_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep);
 }
 template <int MB>
 void go_ho4(const StepParams<float> &p, const HoTab<float> &w, int S, int jstep, cudaStream_t st, bool h, int kz) {
@@ -397,7 +401,7 @@ cudaError_t launch_ho(const StepParams<R> &p, const HoTab<R> &w, int S, int jste
         if (lean_h) {
             if constexpr (sizeof(R) == 4) e = launch_ho4(p, w, S, jstep, st, true, p.KZ_h, p.MB_h);
         } else {
-            k_h_ho<R><<<grid, blk, 0, st>>>(p, w, jstep);
+            launch_pdl(k_h_ho<R>, grid, blk, st, p, w, jstep);
             g_launches++;
         }
     }
@@ -405,7 +409,7 @@ cudaError_t launch_ho(const StepParams<R> &p, const HoTab<R> &w, int S, int jste
         if (lean_e) {
             if constexpr (sizeof(R) == 4) e = launch_ho4(p, w, S, jstep, st, false, p.KZ_e, p.MB_e);
         } else {
-            k_e_ho<R><<<grid, blk, 0, st>>>(p, w, jstep);
+            launch_pdl(k_e_ho<R>, grid, blk, st, p, w, jstep);
             g_launches++;
         }
     }

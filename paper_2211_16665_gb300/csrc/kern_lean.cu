@@ -250,13 +250,14 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepPa
     const int k0 = (blockIdx.z / S) * KZ;         // z block follow one another
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
-    const int n = *p.step + jstep;
     const int vol = (int)p.vol, plane = (int)p.plane, npml = p.npml;
+    LeanRow<W> r;
+    lean_row<W>(p, p.lx, p.ly, true, i, j, r);
+    pdl_wait();
+    const int n = *p.step + jstep;
     const float *__restrict__ E = p.ering + (long long)s * p.ering_stride + (long long)(n % p.nslot) * 3 * p.vol;
     float *__restrict__ H = p.H + (long long)s * 3 * vol;
     float *__restrict__ ps = p.psiL + (long long)s * 12 * vol;
-    LeanRow<W> r;
-    lean_row<W>(p, p.lx, p.ly, true, i, j, r);
     const int j0 = blockIdx.y * kLeanRows;
     const bool yblk = (j0 < npml) || (j0 + kLeanRows > p.ny - npml);
 
@@ -271,16 +272,16 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepPa
     }
 }
 
-// H loads of the E update: through the read-only path, or (CG) from L2 only, for H that
-// other blocks of the same launch wrote (the read-only path and L1 are not coherent with them).
+// H loads of the E update: plain (the H kernel may still run when an E block starts, see pdl_wait), or (CG)
+// from L2 only, for H that other blocks of the same launch wrote (L1 is not coherent with them).
 template <int W, bool CG> __device__ __forceinline__ Vec<W> ldh(const float *p) {
-    if constexpr (!CG) return ldc<W>(p);
+    if constexpr (!CG) return ldw<W>(p);
     Vec<W> r;
     if constexpr (W == 1) r.v[0] = __ldcg(p);
     else { const float2 t = __ldcg(reinterpret_cast<const float2 *>(p)); r.v[0] = t.x; r.v[1] = t.y; }
     return r;
 }
-template <bool CG> __device__ __forceinline__ float ldh1(const float *p) { return CG ? __ldcg(p) : __ldg(p); }
+template <bool CG> __device__ __forceinline__ float ldh1(const float *p) { return CG ? __ldcg(p) : *p; }
 
 // One plane k of the E update; hxm, hym: Hx, Hy of plane k-1 (in), of plane k (out).
 template <int W, bool YZ, bool CG>
@@ -394,6 +395,9 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepPa
     const int k0 = (blockIdx.z / S) * KZ;         // block share the dt/eps reads in L2
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
+    LeanRow<W> r;
+    lean_row<W>(p, p.lx, p.ly, false, i, j, r);
+    pdl_wait();
     const int n = *p.step + jstep;
     const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch, npml = p.npml;
     const float *__restrict__ ring = p.ering + (long long)s * p.ering_stride;
@@ -401,15 +405,13 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepPa
     float *__restrict__ En = const_cast<float *>(ring) + (long long)((n + 1) % p.nslot) * 3 * p.vol;
     const float *__restrict__ H = p.H + (long long)s * 3 * vol;
     float *__restrict__ ps = p.psiL + (long long)s * 12 * vol + 6LL * vol;
-    LeanRow<W> r;
-    lean_row<W>(p, p.lx, p.ly, false, i, j, r);
     const int j0 = blockIdx.y * kLeanRows;
     const bool yblk = (j0 < npml) || (j0 + kLeanRows - 1 > p.ny - npml);
     const bool taps = p.colmap && p.inc && p.tflag[s * p.tflag_stride + j * p.nseg + (i >> 5)];
 
     int idx = k0 * plane + j * pitch + i;
     const int im = (k0 > 0) ? idx - plane : idx;      // clamped on the bottom face
-    Vec<W> hxm = ldc<W>(H + im), hym = ldc<W>(H + vol + im);
+    Vec<W> hxm = ldw<W>(H + im), hym = ldw<W>(H + vol + im);
 #pragma unroll
     for (int kk = 0; kk < KZ; ++kk, idx += plane) {
         const int k = k0 + kk;
@@ -525,6 +527,7 @@ __global__ void k_tap_inc(const StepParams<float> p, const int S, const int nste
     const int u = (int)(t % ntl);
     const int s = (int)((t / ntl) % S);
     const int jstep = (int)(t / ((long long)ntl * S));
+    pdl_wait();
     const int n = *p.step + jstep;
     float v = 0.f;
     if (n < nt) {
@@ -564,8 +567,8 @@ void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool
     const dim3 block(kLeanX, kLeanRows);
     const int nv = (p.nx + W - 1) / W;
     const dim3 grid((nv + kLeanX - 1) / kLeanX, (p.ny + kLeanRows - 1) / kLeanRows, ((p.nz + KZ - 1) / KZ) * S);
-    if (h) k_h_lean<W, KZ, MB><<<grid, block, 0, st>>>(p, jstep);
-    else k_e_lean<W, KZ, MB><<<grid, block, 0, st>>>(p, jstep);
+    if (h) launch_pdl(k_h_lean<W, KZ, MB>, grid, block, st, p, jstep);
+    else launch_pdl(k_e_lean<W, KZ, MB>, grid, block, st, p, jstep);
 }
 template <int W, int MB>
 bool lean_kz(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int kz) {
@@ -614,9 +617,8 @@ cudaError_t launch_step_wave(const StepParams<float> &p, int S, int jstep, cudaS
 cudaError_t launch_tap_inc(const StepParams<float> &p, int S, int nsteps, int nt, cudaStream_t st) {
     const long long n = (long long)nsteps * S * p.inc_ntl;
     if (n <= 0 || !p.inc || !p.itaps) return cudaSuccess;
-    k_tap_inc<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p, S, nsteps, nt);
     g_launches++;
-    return cudaGetLastError();
+    return launch_pdl(k_tap_inc, dim3((unsigned)((n + 255) / 256)), dim3(256), st, p, S, nsteps, nt);
 }
 
 cudaError_t launch_mask_coef(const StepParams<float> &p, const float *cE, float *cEm, cudaStream_t st) {

@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_h(const StepParams<R> p, const
     const int i = t - j * p.pitch;
     if (j >= p.NY || i >= p.NX) return;
     const int s = blockIdx.z;
+    pdl_wait();
     const int n = *p.step + jstep;
     const int k0 = blockIdx.y * KZ;
     const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch;
@@ -150,14 +151,15 @@ __global__ void __launch_bounds__(kBlock, MINB) k_e(const StepParams<R> p, const
     const int i = t - j * p.pitch;
     if (j >= p.NY || i >= p.NX) return;
     const int s = blockIdx.z;
+    pdl_wait();
     const int n = *p.step + jstep;
     const int k0 = blockIdx.y * KZ;
     const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch;
     const R *__restrict__ Eo = eslot(p, s, n);
     R *__restrict__ En = const_cast<R *>(eslot(p, s, n + 1));
-    const R *__restrict__ Hx = p.H + (long long)s * 3 * vol;
-    const R *__restrict__ Hy = Hx + vol;
-    const R *__restrict__ Hz = Hx + 2 * vol;
+    const R *Hx = p.H + (long long)s * 3 * vol;
+    const R *Hy = Hx + vol;
+    const R *Hz = Hx + 2 * vol;
     const R *__restrict__ cEx = p.cE;
     const R *__restrict__ cEy = p.cE + vol;
     const R *__restrict__ cEz = p.cE + 2 * vol;
@@ -177,13 +179,13 @@ __global__ void __launch_bounds__(kBlock, MINB) k_e(const StepParams<R> p, const
     const bool ix_in = (i >= 1 && i < nx), jy_in = (j >= 1 && j < ny);
 
     int idx = k0 * plane + j * pitch + i;
-    R hxm = (k0 > 0) ? ldg(Hx + idx - plane) : R(0);
-    R hym = (k0 > 0) ? ldg(Hy + idx - plane) : R(0);
+    R hxm = (k0 > 0) ? Hx[idx - plane] : R(0);
+    R hym = (k0 > 0) ? Hy[idx - plane] : R(0);
 #pragma unroll
     for (int kk = 0; kk < KZ; ++kk, idx += plane) {
         const int k = k0 + kk;
         if (k >= p.NZ) break;
-        const R hxc = ldg(Hx + idx), hyc = ldg(Hy + idx), hzc = ldg(Hz + idx);
+        const R hxc = Hx[idx], hyc = Hy[idx], hzc = Hz[idx];
         const int szn = slab_node(k, nz, p.npml);
         const R ihz = ldg(p.az.ih_n + k);
         R bz = 0, azc = 0;
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_e(const StepParams<R> p, const
         const bool kz_in = (k >= 1 && k < nz);
 
         if (i < nx && jy_in && kz_in) {   // Ex at (i+1/2, j, k)
-            R dHz_dy = (hzc - ldg(Hz + idx - pitch)) * ihy;
+            R dHz_dy = (hzc - Hz[idx - pitch]) * ihy;
             R dHy_dz = (hyc - hym) * ihz;
             if (syn >= 0) {
                 R &ps = psy[2 * p.sy + (k * np2 + syn) * pitch + i];
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_e(const StepParams<R> p, const
         }
         if (j < ny && ix_in && kz_in) {   // Ey at (i, j+1/2, k)
             R dHx_dz = (hxc - hxm) * ihz;
-            R dHz_dx = (hzc - ldg(Hz + idx - 1)) * ihx;
+            R dHz_dx = (hzc - Hz[idx - 1]) * ihx;
             if (szn >= 0) {
                 R &ps = psz[3 * p.sz + (szn * p.NY + j) * pitch + i];
                 ps = bz * ps + azc * dHx_dz;
@@ -221,8 +223,8 @@ __global__ void __launch_bounds__(kBlock, MINB) k_e(const StepParams<R> p, const
             En[vol + idx] = ldg(Eo + vol + idx) + ldg(cEy + idx) * (dHx_dz - dHz_dx);
         }
         if (k < nz && ix_in && jy_in) {   // Ez at (i, j, k+1/2)
-            R dHy_dx = (hyc - ldg(Hy + idx - 1)) * ihx;
-            R dHx_dy = (hxc - ldg(Hx + idx - pitch)) * ihy;
+            R dHy_dx = (hyc - Hy[idx - 1]) * ihx;
+            R dHx_dy = (hxc - Hx[idx - pitch]) * ihy;
             if (sxn >= 0) {
                 R &ps = psx[3 * p.sx + (k * p.NY + j) * np2 + sxn];
                 ps = bx * ps + axc * dHy_dx;
@@ -809,12 +811,15 @@ cudaError_t launch_dft_bulk(const StepParams<float> &p, const PointParams<float>
     return cudaGetLastError();
 }
 
-__global__ void k_advance(int *step, int by) { *step += by; }
+__global__ void k_advance(int *step, int by) {
+    pdl_wait();
+    *step += by;
+}
 
 template <typename R, int KZ, int MB>
 void launch_hz(const StepParams<R> &p, dim3 grid, int jstep, cudaStream_t st, bool h) {
-    if (h) k_h<R, KZ, MB><<<grid, kBlock, 0, st>>>(p, jstep);
-    else k_e<R, KZ, MB><<<grid, kBlock, 0, st>>>(p, jstep);
+    if (h) launch_pdl(k_h<R, KZ, MB>, grid, dim3(kBlock), st, p, jstep);
+    else launch_pdl(k_e<R, KZ, MB>, grid, dim3(kBlock), st, p, jstep);
 }
 
 template <typename R, int MB>
@@ -882,9 +887,8 @@ cudaError_t launch_dft(const StepParams<R> &p, const PointParams<R> &q, int S, i
 }
 
 cudaError_t launch_advance(int *step, int by, cudaStream_t st) {
-    k_advance<<<1, 1, 0, st>>>(step, by);
     g_launches++;
-    return cudaGetLastError();
+    return launch_pdl(k_advance, dim3(1), dim3(1), st, step, by);
 }
 
 template cudaError_t launch_step<float>(const StepParams<float> &, const PointParams<float> &, int, int, cudaStream_t,
