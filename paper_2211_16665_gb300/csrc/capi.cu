@@ -224,8 +224,11 @@ template <typename R>
 void axis_tab(const csem_ctx *c, int a, csem::AxisTab<R> &t) {
     const R *base = (const R *)c->d_tab;
     long long off = 0;
-    for (int b = 0; b < a; ++b) off += 6LL * (c->ax[b].n + 1);
+    for (int b = 0; b < a; ++b) off += 9LL * (c->ax[b].n + 1);
     const int n = c->ax[a].n;
+    t.c_h = base + off + 6 * (n + 1);
+    t.g_h = base + off + 7 * (n + 1);
+    t.g_n = base + off + 8 * (n + 1);
     t.ih_h = base + off;
     t.ih_n = base + off + (n + 1);
     t.b_h = base + off + 2 * (n + 1);
@@ -299,7 +302,13 @@ int upload_tables(csem_ctx *c) {
         std::vector<R> ih_h(n + 1, R(0)), ih_n(n + 1, R(0)), bh(n + 1, R(0)), ah(n + 1, R(0)), bn(n + 1), an(n + 1);
         for (int i = 0; i < n; ++i) { ih_h[i] = (R)(1.0 / A.h[i]); bh[i] = (R)A.bh[i]; ah[i] = (R)A.ah[i]; }
         for (int i = 0; i <= n; ++i) { ih_n[i] = (R)(1.0 / A.ht[i]); bn[i] = (R)A.bn[i]; an[i] = (R)A.an[i]; }
-        for (auto *v : {&ih_h, &ih_n, &bh, &ah, &bn, &an}) tab.insert(tab.end(), v->begin(), v->end());
+        std::vector<R> ch(n + 1, R(0)), gh(n + 1, R(0)), gn(n + 1);
+        for (int i = 0; i < n; ++i) {
+            ch[i] = (R)(c->dt / kMu0 / A.h[i]);
+            gh[i] = (R)(A.ah[i] * (c->dt / kMu0 / A.h[i]));
+        }
+        for (int i = 0; i <= n; ++i) gn[i] = (R)(A.an[i] / A.ht[i]);
+        for (auto *v : {&ih_h, &ih_n, &bh, &ah, &bn, &an, &ch, &gh, &gn}) tab.insert(tab.end(), v->begin(), v->end());
     }
     TRY(dalloc(c, (R **)&c->d_tab, tab.size() * sizeof(R)));
     CK(cudaMemcpy(c->d_tab, tab.data(), tab.size() * sizeof(R), cudaMemcpyHostToDevice));

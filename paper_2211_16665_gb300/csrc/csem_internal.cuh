@@ -114,6 +114,8 @@ struct AxisTab {          // per-axis stepping tables (device, type R)
     const R *ih_h, *ih_n; // 1/h at half nodes [n], 1/h~ at nodes [n+1]
     const R *b_h, *a_h;   // CPML recursion at half nodes [n]
     const R *b_n, *a_n;   // CPML recursion at nodes [n+1]
+    const R *c_h, *g_h;   // FP64 kernels: dt/(mu0 h) and a dt/(mu0 h) at half nodes [n]
+    const R *g_n;         // FP64 kernels: a/h~ at nodes [n+1]
 };
 
 struct GeoTab {            // per-axis FP32 widths for the fused one-pass step (padded to 16-byte groups)
@@ -238,6 +240,8 @@ bool fz_supported(int by, int mb, int kz);
 // (8,1), (8,2)}, kz planes per z block; reads the masked dt/eps and the slab CPML memory
 cudaError_t launch_step_ws(const StepParams<float> &p, int S, int jstep, cudaStream_t st);
 bool ws_supported(int by, int mb, int kz);
+// FP64 H / E kernels (kern_f64.cu), kz in {1,2,4,8}, mb in {4,6,8}
+cudaError_t launch_field64(const StepParams<double> &p, int S, int jstep, cudaStream_t st, bool h, int kz, int mb);
 // FP32 H / E kernels with four cells per thread (kern_vec.cu), kz in {1,2,4,8}, mb in {4,6}
 // lean FP32 H / E kernels (kern_lean.cu), nx % 4 == 0, w (cells per thread) in {1,2}, kz in {1,2,4},
 // mb (resident 128-thread blocks per SM) in {6,8} for w = 1 and {4,6,8} for w = 2
