@@ -434,6 +434,7 @@ csem::StepParams<R> step_params(csem_ctx *c, bool dft, void *acc) {
     p.ering = (R *)c->d_ering;
     p.ering_stride = (long long)c->nslot * 3 * c->vol;
     p.nslot = c->nslot;
+    p.mslot = csem::slot_magic(c->nt, p.nslot);
     p.psi = (R *)c->d_psi;
     p.psi_stride = c->psi_stride; p.sx = c->sx; p.sy = c->sy; p.sz = c->sz;
     p.cE = (const R *)c->d_cE;
@@ -1184,7 +1185,7 @@ int td_impl(csem_ctx *c, const void *rho, const csem_points *src, const csem_poi
     CK(cudaMemsetAsync(acc, 0, v3 * sizeof(double), st));
 
     csem::StepParams<R> pf = step_params<R>(c, false, nullptr);
-    pf.ering = seg; pf.ering_stride = seg_stride; pf.nslot = C + 1;
+    pf.ering = seg; pf.ering_stride = seg_stride; pf.nslot = C + 1; pf.mslot = csem::slot_magic(nt, C + 1);
     pf.colmap = c->d_colmap; pf.colmap_stride = c->plane;
     pf.tflag = c->d_tflag; pf.tflag_stride = (long long)c->ny * c->nseg;
     pf.inc_ntl = 8;
@@ -1199,7 +1200,7 @@ int td_impl(csem_ctx *c, const void *rho, const csem_points *src, const csem_poi
 
     csem::StepParams<R> pa = step_params<R>(c, false, nullptr);
     pa.H = (R *)(w + P.o_aH); pa.H2 = P.fused ? (R *)(w + P.o_aH2) : pa.H;
-    pa.ering = aring; pa.ering_stride = a_stride; pa.nslot = B + 1;
+    pa.ering = aring; pa.ering_stride = a_stride; pa.nslot = B + 1; pa.mslot = csem::slot_magic(nt, B + 1);
     pa.psi = (R *)(w + P.o_apsi);
     if constexpr (sizeof(R) == 4) pa.psiL = P.lean ? (float *)(w + P.o_apsiL) : nullptr;
     pa.colmap = adst.colmap; pa.colmap_stride = 0;
@@ -1699,7 +1700,7 @@ int csem_create(csem_ctx **out, const csem_grid *g, const csem_opts *o) {
     // FP32: tap increments, padded tables and the masked dt/eps of the lean kernels (fourth order: nx even);
     // second order also the CPML memory of the lean split kernels in 12 volume arrays per source, kept when it
     // fits, and, nx even, the fused one-pass step's per-cell material and widths
-    if (rc == CSEM_OK && c->precision == 32 && (c->order == 2 || c->nx % 2 == 0)) {
+    if (rc == CSEM_OK && c->precision == 32 && (c->order == 2 || (c->nx % 2 == 0 && c->vol < (1LL << 30)))) {
         step(dalloc(c, &c->d_inc, (size_t)kChunk * S * std::max(8, NR * 8) * sizeof(float)));
         step(dalloc(c, &c->d_tapk, (size_t)std::max(S, NR) * 8 * sizeof(int)));
         step(upload_lean_tables(c));
@@ -1720,7 +1721,7 @@ int csem_create(csem_ctx **out, const csem_grid *g, const csem_opts *o) {
         size_t free_b = 0, total_b = 0;
         cudaMemGetInfo(&free_b, &total_b);
         const double need = (double)S * 12 * c->vol * sizeof(float);
-        if (need < 0.25 * (double)free_b) {
+        if (need < 0.25 * (double)free_b && c->vol < (1LL << 30)) {   // the kernels' byte offsets are 32 bits
             step(dalloc(c, &c->d_psiL, (size_t)S * 12 * c->vol * sizeof(float)));
             if (c->nx % 4 == 0) step(dalloc(c, &c->d_wave, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)));
             if (rc == CSEM_OK && c->d_wave && cudaMemset(c->d_wave, 0, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)) != cudaSuccess)

@@ -134,6 +134,7 @@ struct StepParams {
     R *ering;                      // [S][nslot][3][vol]
     long long ering_stride;        // nslot*3*vol
     int nslot;                     // transform block M + 1
+    unsigned mslot;                // ceil(2^32 / nslot) where steps * nslot < 2^32, else 0 (see slot_of)
     R *psi;                        // [S][psi_stride]
     long long psi_stride, sx, sy, sz;
     const R *cE;                   // [3][vol] dt/eps on each E edge
@@ -187,6 +188,22 @@ struct StepParams {
     const double *coef;            // [S][n_emit][J]
     const double *T;               // [nt][J]
 };
+
+// x / d by one multiplication: floor(x m / 2^32) with m = ceil(2^32 / d) is exact while x d < 2^32; m = 0
+// stands for d = 1.  (A division by a run-time value is a subroutine of some twenty instructions; a step
+// kernel's thread had five of them.)
+__host__ __device__ inline unsigned div_magic(unsigned d) { return d <= 1 ? 0u : (unsigned)((0x100000000ull + d - 1) / d); }
+__device__ __forceinline__ unsigned div_by(unsigned x, unsigned m) { return m ? __umulhi(x, m) : x; }
+inline unsigned slot_magic(long long steps, int nslot) {
+    return nslot > 1 && (steps + 1) * nslot < 0x100000000ll ? div_magic((unsigned)nslot) : 0u;
+}
+// ring slot of step n, and the slot after it
+template <typename R> __device__ __forceinline__ int slot_of(const StepParams<R> &p, int n) {
+    return p.mslot ? n - (int)__umulhi((unsigned)n, p.mslot) * p.nslot : n % p.nslot;
+}
+template <typename R> __device__ __forceinline__ int slot_after(const StepParams<R> &p, int slot) {
+    return slot + 1 == p.nslot ? 0 : slot + 1;
+}
 
 struct Tap {                       // one trilinear tap of a point operator (32 bytes)
     long long idx;                 // lattice index inside a component block

@@ -164,6 +164,15 @@ __global__ void __launch_bounds__(kHoX *kHoY) k_e_ho(const StepParams<R> p, cons
 __device__ __forceinline__ float2 f2g(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
 __device__ __forceinline__ float2 f2w(const float *p) { return *reinterpret_cast<const float2 *>(p); }
 __device__ __forceinline__ void f2s(float *p, float2 v) { *reinterpret_cast<float2 *>(p) = v; }
+// at a 32-bit byte offset from a base that is the same for the whole block (one add per access)
+__device__ __forceinline__ const float *at(const float *b, unsigned o) {
+    return reinterpret_cast<const float *>(reinterpret_cast<const char *>(b) + o);
+}
+__device__ __forceinline__ float2 f2g(const float *b, unsigned o) { return f2g(at(b, o)); }
+__device__ __forceinline__ float2 f2w(const float *b, unsigned o) { return f2w(at(b, o)); }
+__device__ __forceinline__ float f1g(const float *b, unsigned o) { return __ldg(at(b, o)); }
+__device__ __forceinline__ float f1w(const float *b, unsigned o) { return *at(b, o); }
+__device__ __forceinline__ void f2s(float *b, unsigned o, float2 v) { f2s(const_cast<float *>(at(b, o)), v); }
 __device__ __forceinline__ float4 f4g(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
 // w . (a, b, c, d) for both cells of the pair
 __device__ __forceinline__ float2 dot4(const float4 &w, float2 a, float2 b, float2 c, float2 d) {
@@ -174,18 +183,18 @@ __device__ __forceinline__ float2 dx5(const float4 &w0, const float4 &w1, float 
                                       float f4) {
     return make_float2(w0.x * f0 + w0.y * f1 + w0.z * f2 + w0.w * f3, w1.x * f1 + w1.y * f2 + w1.z * f3 + w1.w * f4);
 }
-__device__ __forceinline__ void pml2(float2 &d, bool in, float b, float a, float *ps) {
+__device__ __forceinline__ void pml2(float2 &d, bool in, float b, float a, float *ps, unsigned o) {
     if (!in) return;
-    float2 v = f2w(ps);
+    float2 v = f2w(ps, o);
     v.x = b * v.x + a * d.x; v.y = b * v.y + a * d.y;
-    f2s(ps, v);
+    f2s(ps, o, v);
     d.x += v.x; d.y += v.y;
 }
-__device__ __forceinline__ void pml2x(float2 &d, bool in0, bool in1, float2 b, float2 a, float *ps) {
+__device__ __forceinline__ void pml2x(float2 &d, bool in0, bool in1, float2 b, float2 a, float *ps, unsigned o) {
     if (!in0 && !in1) return;
-    float2 v = f2w(ps);
+    float2 v = f2w(ps, o);
     v.x = b.x * v.x + a.x * d.x; v.y = b.y * v.y + a.y * d.y;
-    f2s(ps, v);
+    f2s(ps, o, v);
     d.x += v.x; d.y += v.y;
 }
 __device__ __forceinline__ float3 ho_taps(const int *__restrict__ tk, const float *__restrict__ inc, int k, int2 cm) {
@@ -202,19 +211,19 @@ __device__ __forceinline__ float3 ho_taps(const int *__restrict__ tk, const floa
 }
 
 template <int KZ, int MINB>
-__global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, const HoTab<float> w, const int jstep) {
+__global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, const HoTab<float> w, const int jstep,
+                                                     const unsigned S, const unsigned mS) {
     const int i = (blockIdx.x * 32 + threadIdx.x) * 2;
     const int j = blockIdx.y * 4 + threadIdx.y;
-    const int nkb = (p.nz + KZ - 1) / KZ;
-    const int S = gridDim.z / nkb;
-    const int s = blockIdx.z % S, k0 = (blockIdx.z / S) * KZ;
+    const int zb = (int)div_by(blockIdx.z, mS), s = (int)(blockIdx.z - zb * S), k0 = zb * KZ;
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
     pdl_wait();
-    const int n = *p.step + jstep;
+    const int sl = slot_of(p, *p.step + jstep);
     const int nx = p.nx, ny = p.ny, nz = p.nz, npml = p.npml;
-    const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch;
-    const float *__restrict__ Ex = p.ering + (long long)s * p.ering_stride + (long long)(n % p.nslot) * 3 * p.vol;
+    const long long vol = p.vol;
+    const int plane = (int)p.plane, pitch = p.pitch;
+    const float *__restrict__ Ex = p.ering + (long long)s * p.ering_stride + (long long)sl * 3 * p.vol;
     const float *__restrict__ Ey = Ex + vol;
     const float *__restrict__ Ez = Ex + 2 * vol;
     float *__restrict__ H = p.H + (long long)s * 3 * vol;
@@ -222,8 +231,8 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
     const float cH = p.cH;
     // neighbours, clamped on the lattice: column i-1; rows j-1, j+2 (column i+3 lies in the
     // lattice row or its padding, and only the last half node's zero weight meets it there)
-    const int im = (i > 0) ? -1 : 0;
-    const int jm = (j > 0) ? -pitch : 0, jp2 = (j + 2 <= ny) ? 2 * pitch : (ny - j) * pitch;
+    const unsigned im = (i > 0) ? -4 : 0;
+    const unsigned jm = (j > 0) ? -4 * pitch : 0, jp = 4 * pitch, jp2 = (j + 2 <= ny) ? 8 * pitch : 4 * (ny - j) * pitch;
     const float4 wx0 = f4g(w.wxh + 4 * i), wx1 = f4g(w.wxh + 4 * (i + 1)), wy = f4g(w.wyh + 4 * j);
     const bool xs0 = slab_half(i, nx, npml) >= 0, xs1 = slab_half(i + 1, nx, npml) >= 0;
     const bool ys = slab_half(j, ny, npml) >= 0;
@@ -231,73 +240,73 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
     const float2 ax = make_float2(__ldg(p.lx.a_h + i), __ldg(p.lx.a_h + i + 1));
     const float by = __ldg(p.ly.b_h + j), ay = __ldg(p.ly.a_h + j);
     // z window of Ex, Ey at the thread's cells: planes k-1, k, k+1 (k+2 loaded per step)
-    const int base = j * pitch + i;
+    const unsigned base = 4u * (unsigned)(j * pitch + i), dz = 4u * (unsigned)plane;
     int km = (k0 > 0) ? k0 - 1 : 0;
-    float2 xa = f2g(Ex + km * plane + base), xb = f2g(Ex + k0 * plane + base), xc = f2g(Ex + (k0 + 1) * plane + base);
-    float2 ya = f2g(Ey + km * plane + base), yb = f2g(Ey + k0 * plane + base), yc = f2g(Ey + (k0 + 1) * plane + base);
+    float2 xa = f2g(Ex, km * dz + base), xb = f2g(Ex, k0 * dz + base), xc = f2g(Ex, (k0 + 1) * dz + base);
+    float2 ya = f2g(Ey, km * dz + base), yb = f2g(Ey, k0 * dz + base), yc = f2g(Ey, (k0 + 1) * dz + base);
 #pragma unroll
     for (int kk = 0; kk < KZ; ++kk) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        const int idx = k * plane + base;
+        const unsigned o = k * dz + base;
         const int kp2 = (k + 2 <= nz) ? k + 2 : nz;
-        const float2 xd = f2g(Ex + kp2 * plane + base), yd = f2g(Ey + kp2 * plane + base);
+        const float2 xd = f2g(Ex, kp2 * dz + base), yd = f2g(Ey, kp2 * dz + base);
         const float4 wz = f4g(w.wzh + 4 * k);
         // x neighbours of Ey, Ez (plane k): values at i-1 .. i+3
-        const float eym = __ldg(Ey + idx + im), ezm = __ldg(Ez + idx + im);
-        const float2 ez01 = f2g(Ez + idx), ey23 = f2g(Ey + idx + 2), ez23 = f2g(Ez + idx + 2);
+        const float eym = f1g(Ey, o + im), ezm = f1g(Ez, o + im);
+        const float2 ez01 = f2g(Ez, o), ey23 = f2g(Ey, o + 8), ez23 = f2g(Ez, o + 8);
         // y neighbours of Ex, Ez (plane k): rows j-1, j+1, j+2
-        const float2 exm = f2g(Ex + idx + jm), exp1 = f2g(Ex + idx + pitch), exp2 = f2g(Ex + idx + jp2);
-        const float2 ezm2 = f2g(Ez + idx + jm), ezp1 = f2g(Ez + idx + pitch), ezp2 = f2g(Ez + idx + jp2);
-        float2 hx = f2w(H + idx), hy = f2w(H + vol + idx), hz = f2w(H + 2 * vol + idx);
+        const float2 exm = f2g(Ex, o + jm), exp1 = f2g(Ex, o + jp), exp2 = f2g(Ex, o + jp2);
+        const float2 ezm2 = f2g(Ez, o + jm), ezp1 = f2g(Ez, o + jp), ezp2 = f2g(Ez, o + jp2);
+        float2 hx = f2w(H, o), hy = f2w(H + vol, o), hz = f2w(H + 2 * vol, o);
         float2 dEz_dy = dot4(wy, ezm2, ez01, ezp1, ezp2), dEy_dz = dot4(wz, ya, yb, yc, yd);
         float2 dEx_dz = dot4(wz, xa, xb, xc, xd), dEz_dx = dx5(wx0, wx1, ezm, ez01.x, ez01.y, ez23.x, ez23.y);
         float2 dEy_dx = dx5(wx0, wx1, eym, yb.x, yb.y, ey23.x, ey23.y), dEx_dy = dot4(wy, exm, xb, exp1, exp2);
         const bool zs = slab_half(k, nz, npml) >= 0;
         if (ys || zs || xs0 || xs1) {
             const float bz = __ldg(p.lz.b_h + k), az = __ldg(p.lz.a_h + k);
-            pml2(dEz_dy, ys, by, ay, P + idx);
-            pml2(dEy_dz, zs, bz, az, P + vol + idx);
-            pml2(dEx_dz, zs, bz, az, P + 2 * vol + idx);
-            pml2x(dEz_dx, xs0, xs1, bx, ax, P + 3 * vol + idx);
-            pml2x(dEy_dx, xs0, xs1, bx, ax, P + 4 * vol + idx);
-            pml2(dEx_dy, ys, by, ay, P + 5 * vol + idx);
+            pml2(dEz_dy, ys, by, ay, P, o);
+            pml2(dEy_dz, zs, bz, az, P + vol, o);
+            pml2(dEx_dz, zs, bz, az, P + 2 * vol, o);
+            pml2x(dEz_dx, xs0, xs1, bx, ax, P + 3 * vol, o);
+            pml2x(dEy_dx, xs0, xs1, bx, ax, P + 4 * vol, o);
+            pml2(dEx_dy, ys, by, ay, P + 5 * vol, o);
         }
         hx.x -= cH * (dEz_dy.x - dEy_dz.x); hx.y -= cH * (dEz_dy.y - dEy_dz.y);
         hy.x -= cH * (dEx_dz.x - dEz_dx.x); hy.y -= cH * (dEx_dz.y - dEz_dx.y);
         hz.x -= cH * (dEy_dx.x - dEx_dy.x); hz.y -= cH * (dEy_dx.y - dEx_dy.y);
-        f2s(H + idx, hx);
-        f2s(H + vol + idx, hy);
-        f2s(H + 2 * vol + idx, hz);
+        f2s(H, o, hx);
+        f2s(H + vol, o, hy);
+        f2s(H + 2 * vol, o, hz);
         xa = xb; xb = xc; xc = xd;
         ya = yb; yb = yc; yc = yd;
     }
 }
 
 template <int KZ, int MINB>
-__global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, const HoTab<float> w, const int jstep) {
+__global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, const HoTab<float> w, const int jstep,
+                                                     const unsigned S, const unsigned mS) {
     const int i = (blockIdx.x * 32 + threadIdx.x) * 2;
     const int j = blockIdx.y * 4 + threadIdx.y;
-    const int nkb = (p.nz + KZ - 1) / KZ;
-    const int S = gridDim.z / nkb;
-    const int s = blockIdx.z % S, k0 = (blockIdx.z / S) * KZ;
+    const int zb = (int)div_by(blockIdx.z, mS), s = (int)(blockIdx.z - zb * S), k0 = zb * KZ;
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
     pdl_wait();
-    const int n = *p.step + jstep;
+    const int sl = slot_of(p, *p.step + jstep);
     const int nx = p.nx, ny = p.ny, nz = p.nz, npml = p.npml;
-    const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch;
+    const long long vol = p.vol;
+    const int plane = (int)p.plane, pitch = p.pitch;
     const float *__restrict__ ring = p.ering + (long long)s * p.ering_stride;
-    const float *__restrict__ Eo = ring + (long long)(n % p.nslot) * 3 * p.vol;
-    float *__restrict__ En = const_cast<float *>(ring) + (long long)((n + 1) % p.nslot) * 3 * p.vol;
+    const float *__restrict__ Eo = ring + (long long)sl * 3 * p.vol;
+    float *__restrict__ En = const_cast<float *>(ring) + (long long)slot_after(p, sl) * 3 * p.vol;
     const float *__restrict__ Hx = p.H + (long long)s * 3 * vol;
     const float *__restrict__ Hy = Hx + vol;
     const float *__restrict__ Hz = Hx + 2 * vol;
     float *__restrict__ P = p.psi + (long long)s * p.psi_stride + 6LL * vol;
     const float *__restrict__ cE = p.cEm;
     // neighbours, clamped on the lattice: columns i-2; rows j-2, j-1
-    const int im2 = (i >= 2) ? -2 : -i;
-    const int jm2 = (j >= 2) ? -2 * pitch : -j * pitch, jm1 = (j >= 1) ? -pitch : 0;
+    const unsigned im2 = (i >= 2) ? -8 : -4 * i;
+    const unsigned jm2 = (j >= 2) ? -8 * pitch : -4 * j * pitch, jm1 = (j >= 1) ? -4 * pitch : 0, jp = 4 * pitch;
     const float4 wx0 = f4g(w.wxn + 4 * i), wx1 = f4g(w.wxn + 4 * (i + 1)), wy = f4g(w.wyn + 4 * j);
     const bool xs0 = slab_node(i, nx, npml) >= 0, xs1 = slab_node(i + 1, nx, npml) >= 0;
     const bool ys = slab_node(j, ny, npml) >= 0;
@@ -306,26 +315,26 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
     const float by = __ldg(p.ly.b_n + j), ay = __ldg(p.ly.a_n + j);
     const bool taps = p.colmap && p.inc && p.tflag[s * p.tflag_stride + j * p.nseg + (i >> 5)];
     // z window of Hx, Hy at the thread's cells: planes k-2, k-1, k (k+1 loaded per step)
-    const int base = j * pitch + i;
+    const unsigned base = 4u * (unsigned)(j * pitch + i), dz = 4u * (unsigned)plane;
     const int ka = (k0 >= 2) ? k0 - 2 : 0, kb = (k0 >= 1) ? k0 - 1 : 0;
-    float2 xa = f2w(Hx + ka * plane + base), xb = f2w(Hx + kb * plane + base), xc = f2w(Hx + k0 * plane + base);
-    float2 ya = f2w(Hy + ka * plane + base), yb = f2w(Hy + kb * plane + base), yc = f2w(Hy + k0 * plane + base);
+    float2 xa = f2w(Hx, ka * dz + base), xb = f2w(Hx, kb * dz + base), xc = f2w(Hx, k0 * dz + base);
+    float2 ya = f2w(Hy, ka * dz + base), yb = f2w(Hy, kb * dz + base), yc = f2w(Hy, k0 * dz + base);
 #pragma unroll
     for (int kk = 0; kk < KZ; ++kk) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        const int idx = k * plane + base;
-        const float2 xd = f2w(Hx + idx + plane), yd = f2w(Hy + idx + plane);   // plane k+1 <= nz
+        const unsigned o = k * dz + base;
+        const float2 xd = f2w(Hx, o + dz), yd = f2w(Hy, o + dz);   // plane k+1 <= nz
         const float4 wz = f4g(w.wzn + 4 * k);
         // x neighbours of Hy, Hz (plane k): values at i-2 .. i+2
-        const float2 hym = f2w(Hy + idx + im2), hzm = f2w(Hz + idx + im2);
-        const float2 hz01 = f2w(Hz + idx);
-        const float hy2 = Hy[idx + 2], hz2 = Hz[idx + 2];
+        const float2 hym = f2w(Hy, o + im2), hzm = f2w(Hz, o + im2);
+        const float2 hz01 = f2w(Hz, o);
+        const float hy2 = f1w(Hy, o + 8), hz2 = f1w(Hz, o + 8);
         // y neighbours of Hx, Hz (plane k): rows j-2, j-1, j+1
-        const float2 hxm2 = f2w(Hx + idx + jm2), hxm1 = f2w(Hx + idx + jm1), hxp1 = f2w(Hx + idx + pitch);
-        const float2 hzm2 = f2w(Hz + idx + jm2), hzm1 = f2w(Hz + idx + jm1), hzp1 = f2w(Hz + idx + pitch);
-        const float2 e0 = f2g(Eo + idx), e1 = f2g(Eo + vol + idx), e2 = f2g(Eo + 2 * vol + idx);
-        const float2 c0 = f2g(cE + idx), c1 = f2g(cE + vol + idx), c2 = f2g(cE + 2 * vol + idx);
+        const float2 hxm2 = f2w(Hx, o + jm2), hxm1 = f2w(Hx, o + jm1), hxp1 = f2w(Hx, o + jp);
+        const float2 hzm2 = f2w(Hz, o + jm2), hzm1 = f2w(Hz, o + jm1), hzp1 = f2w(Hz, o + jp);
+        const float2 e0 = f2g(Eo, o), e1 = f2g(Eo + vol, o), e2 = f2g(Eo + 2 * vol, o);
+        const float2 c0 = f2g(cE, o), c1 = f2g(cE + vol, o), c2 = f2g(cE + 2 * vol, o);
         float2 dHz_dy = dot4(wy, hzm2, hzm1, hz01, hzp1), dHy_dz = dot4(wz, ya, yb, yc, yd);
         float2 dHx_dz = dot4(wz, xa, xb, xc, xd);
         float2 dHz_dx = dx5(wx0, wx1, hzm.x, hzm.y, hz01.x, hz01.y, hz2);
@@ -334,12 +343,12 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
         const bool zs = slab_node(k, nz, npml) >= 0;
         if (ys || zs || xs0 || xs1) {
             const float bz = __ldg(p.lz.b_n + k), az = __ldg(p.lz.a_n + k);
-            pml2(dHz_dy, ys, by, ay, P + idx);
-            pml2(dHy_dz, zs, bz, az, P + vol + idx);
-            pml2(dHx_dz, zs, bz, az, P + 2 * vol + idx);
-            pml2x(dHz_dx, xs0, xs1, bx, ax, P + 3 * vol + idx);
-            pml2x(dHy_dx, xs0, xs1, bx, ax, P + 4 * vol + idx);
-            pml2(dHx_dy, ys, by, ay, P + 5 * vol + idx);
+            pml2(dHz_dy, ys, by, ay, P, o);
+            pml2(dHy_dz, zs, bz, az, P + vol, o);
+            pml2(dHx_dz, zs, bz, az, P + 2 * vol, o);
+            pml2x(dHz_dx, xs0, xs1, bx, ax, P + 3 * vol, o);
+            pml2x(dHy_dx, xs0, xs1, bx, ax, P + 4 * vol, o);
+            pml2(dHx_dy, ys, by, ay, P + 5 * vol, o);
         }
         float2 ex = make_float2(e0.x + c0.x * (dHz_dy.x - dHy_dz.x), e0.y + c0.y * (dHz_dy.y - dHy_dz.y));
         float2 ey = make_float2(e1.x + c1.x * (dHx_dz.x - dHz_dx.x), e1.y + c1.y * (dHx_dz.y - dHz_dx.y));
@@ -347,14 +356,14 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
         if (taps) {
             const int2 *cm = p.colmap + (long long)s * p.colmap_stride + j * pitch + i;
             const int *tk = p.tapk + (long long)s * p.itap_stride;
-            const float *inc = p.inc + ((long long)jstep * S + s) * p.inc_ntl;
+            const float *inc = p.inc + ((long long)jstep * (int)S + s) * p.inc_ntl;
             const int2 cc0 = __ldg(cm), cc1 = __ldg(cm + 1);
             if (cc0.y) { const float3 a = ho_taps(tk, inc, k, cc0); ex.x += a.x; ey.x += a.y; ez.x += a.z; }
             if (cc1.y) { const float3 a = ho_taps(tk, inc, k, cc1); ex.y += a.x; ey.y += a.y; ez.y += a.z; }
         }
-        f2s(En + idx, ex);
-        f2s(En + vol + idx, ey);
-        f2s(En + 2 * vol + idx, ez);
+        f2s(En, o, ex);
+        f2s(En + vol, o, ey);
+        f2s(En + 2 * vol, o, ez);
         xa = xb; xb = xc; xc = xd;
         ya = yb; yb = yc; yc = yd;
     }
@@ -363,8 +372,9 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
 template <int KZ, int MB>
 void go_ho4k(const StepParams<float> &p, const HoTab<float> &w, int S, int jstep, cudaStream_t st, bool h) {
     const dim3 grid((unsigned)((p.nx / 2 + 31) / 32), (unsigned)((p.ny + 3) / 4), (unsigned)(((p.nz + KZ - 1) / KZ) * S));
-    if (h) launch_pdl(k_h_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep);
-    else launch_pdl(k_e_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep);
+    const unsigned mS = div_magic((unsigned)S);
+    if (h) launch_pdl(k_h_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS);
+    else launch_pdl(k_e_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS);
 }
 template <int MB>
 void go_ho4(const StepParams<float> &p, const HoTab<float> &w, int S, int jstep, cudaStream_t st, bool h, int kz) {

@@ -55,6 +55,21 @@ template <int W> __device__ __forceinline__ void stv(float *p, const Vec<W> &a) 
     if constexpr (W == 1) *p = a.v[0];
     else *reinterpret_cast<float2 *>(p) = make_float2(a.v[0], a.v[1]);
 }
+// The same at a byte offset (32 bits, unsigned) from a base that is the same for the whole block: the base stays
+// in uniform registers and an access costs one add for its offset, where a 64-bit index per access took three to
+// four.  An offset reaches 4 GB, a component of 2^30 entries.
+template <int W> __device__ __forceinline__ Vec<W> ldc(const float *b, unsigned o) {
+    return ldc<W>(reinterpret_cast<const float *>(reinterpret_cast<const char *>(b) + o));
+}
+template <int W> __device__ __forceinline__ Vec<W> ldw(const float *b, unsigned o) {
+    return ldw<W>(reinterpret_cast<const float *>(reinterpret_cast<const char *>(b) + o));
+}
+template <int W> __device__ __forceinline__ void stv(float *b, unsigned o, const Vec<W> &a) {
+    stv<W>(reinterpret_cast<float *>(reinterpret_cast<char *>(b) + o), a);
+}
+__device__ __forceinline__ float ldc1(const float *b, unsigned o) {
+    return __ldg(reinterpret_cast<const float *>(reinterpret_cast<const char *>(b) + o));
+}
 template <int W> __device__ __forceinline__ Vec<W> zv() {
     Vec<W> r;
 #pragma unroll
@@ -118,6 +133,9 @@ template <int W> struct LeanRow {
     bool xs, ys;
     Vec<W> ihx, bx, ax;
     float ihy, by, ay;
+    __device__ __forceinline__ unsigned xoff(const StepParams<float> &p, int k) const {   // bytes, plane k
+        return 4u * (unsigned)((k * p.ny + j) * nxs + ixs);
+    }
 };
 template <int W>
 __device__ __forceinline__ void lean_row(const StepParams<float> &p, const AxisTab<float> &tx, const AxisTab<float> &ty,
@@ -156,22 +174,26 @@ __device__ __forceinline__ float3 lean_taps(const int *__restrict__ tk, const fl
 }  // namespace
 
 // One plane k of the H update for the thread's W cells; YZ: the y/z recursion
-// may apply (a block on a y or z slab).  exc, eyc: Ex, Ey of plane k (in), of
-// plane k+1 (out).
+// may apply (a block on a y or z slab).  o: byte offset of the cells in a component,
+// xo: of their x-slab entries.  exc, eyc: Ex, Ey of plane k (in), of plane k+1 (out).
 template <int W, bool YZ>
 __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float *__restrict__ E, float *__restrict__ H,
-                                        float *__restrict__ ps, const LeanRow<W> &r, int k, int idx, Vec<W> &exc,
-                                        Vec<W> &eyc) {
-    const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch, npml = p.npml;
-    const Vec<W> ezc = ldc<W>(E + 2 * vol + idx);
-    const Vec<W> exk = ldc<W>(E + idx + plane), eyk = ldc<W>(E + vol + idx + plane);
-    const Vec<W> exj = ldc<W>(E + idx + pitch), ezj = ldc<W>(E + 2 * vol + idx + pitch);
-    const float eyn = __ldg(E + vol + idx + W), ezn = __ldg(E + 2 * vol + idx + W);
+                                        float *__restrict__ ps, const LeanRow<W> &r, int k, unsigned o, unsigned xo,
+                                        Vec<W> &exc, Vec<W> &eyc) {
+    const long long vol = p.vol;
+    const unsigned plane = 4u * (unsigned)p.plane, pitch = 4u * (unsigned)p.pitch;
+    const int npml = p.npml;
+    const float *Ey = E + vol, *Ez = E + 2 * vol;
+    float *Hy = H + vol, *Hz = H + 2 * vol;
+    const Vec<W> ezc = ldc<W>(Ez, o);
+    const Vec<W> exk = ldc<W>(E, o + plane), eyk = ldc<W>(Ey, o + plane);
+    const Vec<W> exj = ldc<W>(E, o + pitch), ezj = ldc<W>(Ez, o + pitch);
+    const float eyn = ldc1(Ey, o + 4u * W), ezn = ldc1(Ez, o + 4u * W);
     const float ihz = __ldg(p.lz.ih_h + k);
-    Vec<W> hx = ldw<W>(H + idx), hy = ldw<W>(H + vol + idx), hz = ldw<W>(H + 2 * vol + idx);
-    const int xo = (k * p.ny + r.j) * r.nxs + r.ixs;
-    float *px3 = ps + 3 * vol + xo, *px4 = ps + 4 * vol + xo;
-    Vec<W> q3 = ldw<W>(r.xs ? px3 : p.lzero), q4 = ldw<W>(r.xs ? px4 : p.lzero);
+    Vec<W> hx = ldw<W>(H, o), hy = ldw<W>(Hy, o), hz = ldw<W>(Hz, o);
+    float *px3 = ps + 3 * vol, *px4 = ps + 4 * vol;
+    Vec<W> q3 = zv<W>(), q4 = zv<W>();
+    if (r.xs) { q3 = ldw<W>(px3, xo); q4 = ldw<W>(px4, xo); }
     bool zs = false, ys = false;
     float bz = 0.f, az = 0.f;
     Vec<W> q0 = zv<W>(), q1 = zv<W>(), q2 = zv<W>(), q5 = zv<W>();
@@ -179,32 +201,32 @@ __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float 
         zs = (k < npml) || (k >= p.nz - npml);
         ys = r.ys;
         if (zs) { bz = __ldg(p.lz.b_h + k); az = __ldg(p.lz.a_h + k); }
-        if (ys) { q0 = ldw<W>(ps + idx); q5 = ldw<W>(ps + 5 * vol + idx); }
-        if (zs) { q1 = ldw<W>(ps + vol + idx); q2 = ldw<W>(ps + 2 * vol + idx); }
+        if (ys) { q0 = ldw<W>(ps, o); q5 = ldw<W>(ps + 5 * vol, o); }
+        if (zs) { q1 = ldw<W>(ps + vol, o); q2 = ldw<W>(ps + 2 * vol, o); }
     }
     const Vec<W> ezx = up<W>(ezc, ezn), eyx = up<W>(eyc, eyn);   // Ez, Ey at i+1 .. i+W
 
     // Hx at (i, j+1/2, k+1/2)
     Vec<W> dEz_dy = dsc<W>(ezj, ezc, r.ihy), dEy_dz = dsc<W>(eyk, eyc, ihz);
-    if (YZ && ys) { cpml<W>(q0, dEz_dy, r.by, r.ay); stv<W>(ps + idx, q0); }
-    if (YZ && zs) { cpml<W>(q1, dEy_dz, bz, az); stv<W>(ps + vol + idx, q1); }
+    if (YZ && ys) { cpml<W>(q0, dEz_dy, r.by, r.ay); stv<W>(ps, o, q0); }
+    if (YZ && zs) { cpml<W>(q1, dEy_dz, bz, az); stv<W>(ps + vol, o, q1); }
     hsub<W>(hx, p.cH, dEz_dy, dEy_dz);
     // Hy at (i+1/2, j, k+1/2)
     Vec<W> dEx_dz = dsc<W>(exk, exc, ihz), dEz_dx = dsc<W>(ezx, ezc, r.ihx);
-    if (YZ && zs) { cpml<W>(q2, dEx_dz, bz, az); stv<W>(ps + 2 * vol + idx, q2); }
+    if (YZ && zs) { cpml<W>(q2, dEx_dz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
     cpml<W>(q3, dEz_dx, r.bx, r.ax);
-    if (r.xs) stv<W>(px3, q3);
+    if (r.xs) stv<W>(px3, xo, q3);
     hsub<W>(hy, p.cH, dEx_dz, dEz_dx);
     // Hz at (i+1/2, j+1/2, k)
     Vec<W> dEy_dx = dsc<W>(eyx, eyc, r.ihx), dEx_dy = dsc<W>(exj, exc, r.ihy);
     cpml<W>(q4, dEy_dx, r.bx, r.ax);
-    if (r.xs) stv<W>(px4, q4);
-    if (YZ && ys) { cpml<W>(q5, dEx_dy, r.by, r.ay); stv<W>(ps + 5 * vol + idx, q5); }
+    if (r.xs) stv<W>(px4, xo, q4);
+    if (YZ && ys) { cpml<W>(q5, dEx_dy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
     hsub<W>(hz, p.cH, dEy_dx, dEx_dy);
 
-    stv<W>(H + idx, hx);
-    stv<W>(H + vol + idx, hy);
-    stv<W>(H + 2 * vol + idx, hz);
+    stv<W>(H, o, hx);
+    stv<W>(Hy, o, hy);
+    stv<W>(Hz, o, hz);
     exc = exk;
     eyc = eyk;
 }
@@ -219,9 +241,10 @@ __device__ __forceinline__ void h_tile(const StepParams<float> &p, const int jst
     const int k0 = kb * KZ;
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
-    const int n = *p.step + jstep;
-    const int vol = (int)p.vol, plane = (int)p.plane, npml = p.npml;
-    const float *__restrict__ E = p.ering + (long long)s * p.ering_stride + (long long)(n % p.nslot) * 3 * p.vol;
+    const int sl = slot_of(p, *p.step + jstep);
+    const int plane = (int)p.plane, npml = p.npml;
+    const long long vol = p.vol;
+    const float *__restrict__ E = p.ering + (long long)s * p.ering_stride + (long long)sl * 3 * p.vol;
     float *__restrict__ H = p.H + (long long)s * 3 * vol;
     float *__restrict__ ps = p.psiL + (long long)s * 12 * vol;
     LeanRow<W> r;
@@ -229,78 +252,86 @@ __device__ __forceinline__ void h_tile(const StepParams<float> &p, const int jst
     const int j0 = yb * kLeanRows;
     const bool yblk = (j0 < npml) || (j0 + kLeanRows > p.ny - npml);
 
-    int idx = k0 * plane + j * p.pitch + i;
-    Vec<W> exc = ldc<W>(E + idx), eyc = ldc<W>(E + vol + idx);
+    unsigned o = 4u * (unsigned)(k0 * plane + j * p.pitch + i), xo = r.xoff(p, k0);
+    const unsigned dx = 4u * (unsigned)(p.ny * r.nxs);
+    Vec<W> exc = ldc<W>(E, o), eyc = ldc<W>(E + p.vol, o);
 #pragma unroll
-    for (int kk = 0; kk < KZ; ++kk, idx += plane) {
+    for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true>(p, E, H, ps, r, k, idx, exc, eyc);
-        else h_plane<W, false>(p, E, H, ps, r, k, idx, exc, eyc);
+        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true>(p, E, H, ps, r, k, o, xo, exc, eyc);
+        else h_plane<W, false>(p, E, H, ps, r, k, o, xo, exc, eyc);
     }
 }
 
 template <int W, int KZ, int MINB>
-__global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepParams<float> p, const int jstep) {
+__global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepParams<float> p, const int jstep, const unsigned S,
+                                                                       const unsigned mS) {
     const int i = (blockIdx.x * kLeanX + threadIdx.x) * W;
     const int j = blockIdx.y * kLeanRows + threadIdx.y;
-    const int nkb = (p.nz + KZ - 1) / KZ;
-    const int S = gridDim.z / nkb;
-    const int s = blockIdx.z % S;                 // the source runs fastest: the sources of one
-    const int k0 = (blockIdx.z / S) * KZ;         // z block follow one another
+    const int zb = (int)div_by(blockIdx.z, mS);   // the source runs fastest: the sources of one
+    const int s = (int)(blockIdx.z - zb * S), k0 = zb * KZ;    // z block follow one another
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
-    const int vol = (int)p.vol, plane = (int)p.plane, npml = p.npml;
+    const int plane = (int)p.plane, npml = p.npml;
+    const long long vol = p.vol;
     LeanRow<W> r;
     lean_row<W>(p, p.lx, p.ly, true, i, j, r);
     pdl_wait();
-    const int n = *p.step + jstep;
-    const float *__restrict__ E = p.ering + (long long)s * p.ering_stride + (long long)(n % p.nslot) * 3 * p.vol;
+    const int sl = slot_of(p, *p.step + jstep);
+    const float *__restrict__ E = p.ering + (long long)s * p.ering_stride + (long long)sl * 3 * p.vol;
     float *__restrict__ H = p.H + (long long)s * 3 * vol;
     float *__restrict__ ps = p.psiL + (long long)s * 12 * vol;
     const int j0 = blockIdx.y * kLeanRows;
     const bool yblk = (j0 < npml) || (j0 + kLeanRows > p.ny - npml);
 
-    int idx = k0 * plane + j * p.pitch + i;
-    Vec<W> exc = ldc<W>(E + idx), eyc = ldc<W>(E + vol + idx);
+    unsigned o = 4u * (unsigned)(k0 * plane + j * p.pitch + i), xo = r.xoff(p, k0);
+    const unsigned dx = 4u * (unsigned)(p.ny * r.nxs);
+    Vec<W> exc = ldc<W>(E, o), eyc = ldc<W>(E + p.vol, o);
 #pragma unroll
-    for (int kk = 0; kk < KZ; ++kk, idx += plane) {
+    for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true>(p, E, H, ps, r, k, idx, exc, eyc);
-        else h_plane<W, false>(p, E, H, ps, r, k, idx, exc, eyc);
+        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true>(p, E, H, ps, r, k, o, xo, exc, eyc);
+        else h_plane<W, false>(p, E, H, ps, r, k, o, xo, exc, eyc);
     }
 }
 
 // H loads of the E update: plain (the H kernel may still run when an E block starts, see pdl_wait), or (CG)
 // from L2 only, for H that other blocks of the same launch wrote (L1 is not coherent with them).
-template <int W, bool CG> __device__ __forceinline__ Vec<W> ldh(const float *p) {
-    if constexpr (!CG) return ldw<W>(p);
+template <int W, bool CG> __device__ __forceinline__ Vec<W> ldh(const float *b, unsigned o) {
+    if constexpr (!CG) return ldw<W>(b, o);
+    const float *p = reinterpret_cast<const float *>(reinterpret_cast<const char *>(b) + o);
     Vec<W> r;
     if constexpr (W == 1) r.v[0] = __ldcg(p);
     else { const float2 t = __ldcg(reinterpret_cast<const float2 *>(p)); r.v[0] = t.x; r.v[1] = t.y; }
     return r;
 }
-template <bool CG> __device__ __forceinline__ float ldh1(const float *p) { return CG ? __ldcg(p) : *p; }
+template <bool CG> __device__ __forceinline__ float ldh1(const float *b, unsigned o) {
+    const float *p = reinterpret_cast<const float *>(reinterpret_cast<const char *>(b) + o);
+    return CG ? __ldcg(p) : *p;
+}
 
-// One plane k of the E update; hxm, hym: Hx, Hy of plane k-1 (in), of plane k (out).
+// One plane k of the E update; o, xo as in h_plane; oj, oi: from o to the lower neighbours along y and x (0 on
+// the outer faces).  hxm, hym: Hx, Hy of plane k-1 (in), of plane k (out).
 template <int W, bool YZ, bool CG>
 __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float *__restrict__ Eo, float *__restrict__ En,
                                         const float *__restrict__ H, float *__restrict__ ps, const LeanRow<W> &r, int s,
-                                        int S, int jstep, int k, int idx, bool taps, Vec<W> &hxm, Vec<W> &hym) {
-    const int vol = (int)p.vol, pitch = p.pitch, npml = p.npml;
+                                        int S, int jstep, int k, unsigned o, unsigned xo, unsigned oj, unsigned oi,
+                                        bool taps, Vec<W> &hxm, Vec<W> &hym) {
+    const long long vol = p.vol;
+    const int npml = p.npml;
     const float *__restrict__ cE = p.cEm;
-    const int ij = (r.j > 0) ? idx - pitch : idx;    // lower neighbours, clamped on the outer faces
-    const int ii = (r.i > 0) ? idx - 1 : idx;
-    const Vec<W> hxc = ldh<W, CG>(H + idx), hyc = ldh<W, CG>(H + vol + idx), hzc = ldh<W, CG>(H + 2 * vol + idx);
-    const Vec<W> hxj = ldh<W, CG>(H + ij), hzj = ldh<W, CG>(H + 2 * vol + ij);
-    const float hyp = ldh1<CG>(H + vol + ii), hzp = ldh1<CG>(H + 2 * vol + ii);
-    const Vec<W> eo0 = ldc<W>(Eo + idx), eo1 = ldc<W>(Eo + vol + idx), eo2 = ldc<W>(Eo + 2 * vol + idx);
-    const Vec<W> c0 = ldc<W>(cE + idx), c1 = ldc<W>(cE + vol + idx), c2 = ldc<W>(cE + 2 * vol + idx);
+    const float *Hy = H + vol, *Hz = H + 2 * vol;
+    const Vec<W> hxc = ldh<W, CG>(H, o), hyc = ldh<W, CG>(Hy, o), hzc = ldh<W, CG>(Hz, o);
+    const Vec<W> hxj = ldh<W, CG>(H, o - oj), hzj = ldh<W, CG>(Hz, o - oj);
+    const float hyp = ldh1<CG>(Hy, o - oi), hzp = ldh1<CG>(Hz, o - oi);
+    const Vec<W> eo0 = ldc<W>(Eo, o), eo1 = ldc<W>(Eo + vol, o), eo2 = ldc<W>(Eo + 2 * vol, o);
+    const Vec<W> c0 = ldc<W>(cE, o), c1 = ldc<W>(cE + vol, o), c2 = ldc<W>(cE + 2 * vol, o);
     const float ihz = __ldg(p.lz.ih_n + k);
-    const int xo = (k * p.ny + r.j) * r.nxs + r.ixs;
-    float *px3 = ps + 3 * vol + xo, *px4 = ps + 4 * vol + xo;
-    Vec<W> q3 = ldw<W>(r.xs ? px3 : p.lzero), q4 = ldw<W>(r.xs ? px4 : p.lzero);
+    float *px3 = ps + 3 * vol, *px4 = ps + 4 * vol;
+    Vec<W> q3 = zv<W>(), q4 = zv<W>();
+    if (r.xs) { q3 = ldw<W>(px3, xo); q4 = ldw<W>(px4, xo); }
     bool zs = false, ys = false;
     float bz = 0.f, az = 0.f;
     Vec<W> q0 = zv<W>(), q1 = zv<W>(), q2 = zv<W>(), q5 = zv<W>();
@@ -308,31 +339,31 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
         zs = (k < npml) || (k > p.nz - npml);
         ys = r.ys;
         if (zs) { bz = __ldg(p.lz.b_n + k); az = __ldg(p.lz.a_n + k); }
-        if (ys) { q0 = ldw<W>(ps + idx); q5 = ldw<W>(ps + 5 * vol + idx); }
-        if (zs) { q1 = ldw<W>(ps + vol + idx); q2 = ldw<W>(ps + 2 * vol + idx); }
+        if (ys) { q0 = ldw<W>(ps, o); q5 = ldw<W>(ps + 5 * vol, o); }
+        if (zs) { q1 = ldw<W>(ps + vol, o); q2 = ldw<W>(ps + 2 * vol, o); }
     }
     const Vec<W> hzx = down<W>(hzp, hzc), hyx = down<W>(hyp, hyc);   // Hz, Hy at i-1 .. i+W-2
 
     // Ex at (i+1/2, j, k)
     Vec<W> dHz_dy = dsc<W>(hzc, hzj, r.ihy), dHy_dz = dsc<W>(hyc, hym, ihz);
-    if (YZ && ys) { cpml<W>(q0, dHz_dy, r.by, r.ay); stv<W>(ps + idx, q0); }
-    if (YZ && zs) { cpml<W>(q1, dHy_dz, bz, az); stv<W>(ps + vol + idx, q1); }
+    if (YZ && ys) { cpml<W>(q0, dHz_dy, r.by, r.ay); stv<W>(ps, o, q0); }
+    if (YZ && zs) { cpml<W>(q1, dHy_dz, bz, az); stv<W>(ps + vol, o, q1); }
     Vec<W> e0 = eadv<W>(eo0, c0, dHz_dy, dHy_dz);
     // Ey at (i, j+1/2, k)
     Vec<W> dHx_dz = dsc<W>(hxc, hxm, ihz), dHz_dx = dsc<W>(hzc, hzx, r.ihx);
-    if (YZ && zs) { cpml<W>(q2, dHx_dz, bz, az); stv<W>(ps + 2 * vol + idx, q2); }
+    if (YZ && zs) { cpml<W>(q2, dHx_dz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
     cpml<W>(q3, dHz_dx, r.bx, r.ax);
-    if (r.xs) stv<W>(px3, q3);
+    if (r.xs) stv<W>(px3, xo, q3);
     Vec<W> e1 = eadv<W>(eo1, c1, dHx_dz, dHz_dx);
     // Ez at (i, j, k+1/2)
     Vec<W> dHy_dx = dsc<W>(hyc, hyx, r.ihx), dHx_dy = dsc<W>(hxc, hxj, r.ihy);
     cpml<W>(q4, dHy_dx, r.bx, r.ax);
-    if (r.xs) stv<W>(px4, q4);
-    if (YZ && ys) { cpml<W>(q5, dHx_dy, r.by, r.ay); stv<W>(ps + 5 * vol + idx, q5); }
+    if (r.xs) stv<W>(px4, xo, q4);
+    if (YZ && ys) { cpml<W>(q5, dHx_dy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
     Vec<W> e2 = eadv<W>(eo2, c2, dHy_dx, dHx_dy);
 
     if (taps) {
-        const int2 *cm = p.colmap + (long long)s * p.colmap_stride + r.j * pitch + r.i;
+        const int2 *cm = p.colmap + (long long)s * p.colmap_stride + r.j * p.pitch + r.i;
         const int *tk = p.tapk + (long long)s * p.itap_stride;
         const float *inc = p.inc + ((long long)jstep * S + s) * p.inc_ntl;
         for (int e = 0; e < W; ++e) {
@@ -342,9 +373,9 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
             e0.v[e] += a.x; e1.v[e] += a.y; e2.v[e] += a.z;
         }
     }
-    stv<W>(En + idx, e0);
-    stv<W>(En + vol + idx, e1);
-    stv<W>(En + 2 * vol + idx, e2);
+    stv<W>(En, o, e0);
+    stv<W>(En + vol, o, e1);
+    stv<W>(En + 2 * vol, o, e2);
     hxm = hxc;
     hym = hyc;
 }
@@ -359,65 +390,68 @@ __device__ __forceinline__ void e_tile(const StepParams<float> &p, const int jst
     const int k0 = kb * KZ;
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
-    const int n = *p.step + jstep;
-    const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch, npml = p.npml;
+    const int sl = slot_of(p, *p.step + jstep);
+    const int plane = (int)p.plane, pitch = p.pitch, npml = p.npml;
+    const long long vol = p.vol;
     const float *__restrict__ ring = p.ering + (long long)s * p.ering_stride;
-    const float *__restrict__ Eo = ring + (long long)(n % p.nslot) * 3 * p.vol;
-    float *__restrict__ En = const_cast<float *>(ring) + (long long)((n + 1) % p.nslot) * 3 * p.vol;
+    const float *__restrict__ Eo = ring + (long long)sl * 3 * p.vol;
+    float *__restrict__ En = const_cast<float *>(ring) + (long long)slot_after(p, sl) * 3 * p.vol;
     const float *__restrict__ H = p.H + (long long)s * 3 * vol;
-    float *__restrict__ ps = p.psiL + (long long)s * 12 * vol + 6LL * vol;
+    float *__restrict__ ps = p.psiL + (long long)s * 12 * vol + 6 * vol;
     LeanRow<W> r;
     lean_row<W>(p, p.lx, p.ly, false, i, j, r);
     const int j0 = yb * kLeanRows;
     const bool yblk = (j0 < npml) || (j0 + kLeanRows - 1 > p.ny - npml);
     const bool taps = p.colmap && p.inc && p.tflag[s * p.tflag_stride + j * p.nseg + (i >> 5)];
 
-    int idx = k0 * plane + j * pitch + i;
-    const int im = (k0 > 0) ? idx - plane : idx;      // clamped on the bottom face
-    Vec<W> hxm = ldh<W, CG>(H + im), hym = ldh<W, CG>(H + vol + im);
+    unsigned o = 4u * (unsigned)(k0 * plane + j * pitch + i), xo = r.xoff(p, k0);
+    const unsigned dx = 4u * (unsigned)(p.ny * r.nxs), oj = j > 0 ? 4u * (unsigned)pitch : 0u, oi = i > 0 ? 4u : 0u;
+    const unsigned om = (k0 > 0) ? o - 4u * (unsigned)plane : o;      // clamped on the bottom face
+    Vec<W> hxm = ldh<W, CG>(H, om), hym = ldh<W, CG>(H + p.vol, om);
 #pragma unroll
-    for (int kk = 0; kk < KZ; ++kk, idx += plane) {
+    for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
         if (yblk || k < npml || k > p.nz - npml)
-            e_plane<W, true, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, idx, taps, hxm, hym);
-        else e_plane<W, false, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, idx, taps, hxm, hym);
+            e_plane<W, true, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, o, xo, oj, oi, taps, hxm, hym);
+        else e_plane<W, false, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, o, xo, oj, oi, taps, hxm, hym);
     }
 }
 
 template <int W, int KZ, int MINB>
-__global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepParams<float> p, const int jstep) {
+__global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepParams<float> p, const int jstep, const unsigned S,
+                                                                       const unsigned mS) {
     const int i = (blockIdx.x * kLeanX + threadIdx.x) * W;
     const int j = blockIdx.y * kLeanRows + threadIdx.y;
-    const int nkb = (p.nz + KZ - 1) / KZ;
-    const int S = gridDim.z / nkb;
-    const int s = blockIdx.z % S;                 // the source runs fastest: the sources of one z
-    const int k0 = (blockIdx.z / S) * KZ;         // block share the dt/eps reads in L2
+    const int zb = (int)div_by(blockIdx.z, mS);   // the source runs fastest: the sources of one z
+    const int s = (int)(blockIdx.z - zb * S), k0 = zb * KZ;    // block share the dt/eps reads in L2
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
     LeanRow<W> r;
     lean_row<W>(p, p.lx, p.ly, false, i, j, r);
     pdl_wait();
-    const int n = *p.step + jstep;
-    const int vol = (int)p.vol, plane = (int)p.plane, pitch = p.pitch, npml = p.npml;
+    const int sl = slot_of(p, *p.step + jstep);
+    const int plane = (int)p.plane, pitch = p.pitch, npml = p.npml;
+    const long long vol = p.vol;
     const float *__restrict__ ring = p.ering + (long long)s * p.ering_stride;
-    const float *__restrict__ Eo = ring + (long long)(n % p.nslot) * 3 * p.vol;
-    float *__restrict__ En = const_cast<float *>(ring) + (long long)((n + 1) % p.nslot) * 3 * p.vol;
+    const float *__restrict__ Eo = ring + (long long)sl * 3 * p.vol;
+    float *__restrict__ En = const_cast<float *>(ring) + (long long)slot_after(p, sl) * 3 * p.vol;
     const float *__restrict__ H = p.H + (long long)s * 3 * vol;
-    float *__restrict__ ps = p.psiL + (long long)s * 12 * vol + 6LL * vol;
+    float *__restrict__ ps = p.psiL + (long long)s * 12 * vol + 6 * vol;
     const int j0 = blockIdx.y * kLeanRows;
     const bool yblk = (j0 < npml) || (j0 + kLeanRows - 1 > p.ny - npml);
     const bool taps = p.colmap && p.inc && p.tflag[s * p.tflag_stride + j * p.nseg + (i >> 5)];
 
-    int idx = k0 * plane + j * pitch + i;
-    const int im = (k0 > 0) ? idx - plane : idx;      // clamped on the bottom face
-    Vec<W> hxm = ldw<W>(H + im), hym = ldw<W>(H + vol + im);
+    unsigned o = 4u * (unsigned)(k0 * plane + j * pitch + i), xo = r.xoff(p, k0);
+    const unsigned dx = 4u * (unsigned)(p.ny * r.nxs), oj = j > 0 ? 4u * (unsigned)pitch : 0u, oi = i > 0 ? 4u : 0u;
+    const unsigned om = (k0 > 0) ? o - 4u * (unsigned)plane : o;      // clamped on the bottom face
+    Vec<W> hxm = ldh<W, false>(H, om), hym = ldh<W, false>(H + p.vol, om);
 #pragma unroll
-    for (int kk = 0; kk < KZ; ++kk, idx += plane) {
+    for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        if (yblk || k < npml || k > p.nz - npml) e_plane<W, true, false>(p, Eo, En, H, ps, r, s, S, jstep, k, idx, taps, hxm, hym);
-        else e_plane<W, false, false>(p, Eo, En, H, ps, r, s, S, jstep, k, idx, taps, hxm, hym);
+        if (yblk || k < npml || k > p.nz - npml) e_plane<W, true, false>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, o, xo, oj, oi, taps, hxm, hym);
+        else e_plane<W, false, false>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, o, xo, oj, oi, taps, hxm, hym);
     }
 }
 
@@ -567,8 +601,9 @@ void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool
     const dim3 block(kLeanX, kLeanRows);
     const int nv = (p.nx + W - 1) / W;
     const dim3 grid((nv + kLeanX - 1) / kLeanX, (p.ny + kLeanRows - 1) / kLeanRows, ((p.nz + KZ - 1) / KZ) * S);
-    if (h) launch_pdl(k_h_lean<W, KZ, MB>, grid, block, st, p, jstep);
-    else launch_pdl(k_e_lean<W, KZ, MB>, grid, block, st, p, jstep);
+    const unsigned mS = div_magic((unsigned)S);
+    if (h) launch_pdl(k_h_lean<W, KZ, MB>, grid, block, st, p, jstep, (unsigned)S, mS);
+    else launch_pdl(k_e_lean<W, KZ, MB>, grid, block, st, p, jstep, (unsigned)S, mS);
 }
 template <int W, int MB>
 bool lean_kz(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int kz) {
