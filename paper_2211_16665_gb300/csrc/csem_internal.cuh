@@ -52,6 +52,19 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// Order of the E blocks and eviction of H by the bytes of a step's fields (E^n, E^{n+1}, H of every source, dt/eps).
+// Above kFarBytes they do not stay in the 126 MB L2 from one kernel to the next, and with both kernels walking z
+// upwards each found the planes it starts with evicted by those the other one ended with.  There the E blocks walk z
+// downwards, so each kernel starts with the planes that the one before it touched last, and H is stored with
+// evict_last, which keeps H rather than the CPML memory and the E^n that are not read again soon.  Below it the
+// order does not matter (the fields stay in L2) and the policy costs more than it gives.
+// Forward runs of 256 steps, upwards / downwards with the policy: 77 MB (128 x 128 x 96) 6.80 / 6.95 ms, 103 MB
+// (148 x 148 x 96) 10.5 / 10.4, 133 MB 13.5 / 12.6, 166 MB 16.2 / 14.5, 250 MB (four sources of 116^3) 31.3 / 28.8,
+// 700 MB (two of 256 x 256 x 128) 70.0 / 68.4 (downwards alone 68.7).  The fourth-order kernels take the order only:
+// two sources of 128 x 128 x 96 20.9 / 20.0 ms, 208 x 208 x 96 25.5 / 24.3.
+constexpr long long kFarBytes = 90LL << 20;
+inline bool far_fields(long long vol, int S) { return 12LL * vol * (3 * S + 1) > kFarBytes; }
+
 // Bounded wait on an mbarrier phase, shared by the bulk-copy kernels: true once the phase of
 // this parity has completed; false after about kWaitNs of the global timer (or 2^26 polls),
 // so a kernel whose copies never arrive reports a timeout instead of hanging.

@@ -35,11 +35,11 @@ __device__ __forceinline__ R d_node(const R *F, long long at, long long s, int p
     return d;
 }
 
-// psi <- b psi + a d inside the slab, d + psi returned
+// psi <- b psi + a d inside the slab, d + psi returned; q: psi, loaded with the others of the plane (see pml2)
 template <typename R>
-__device__ __forceinline__ R pml(R d, bool in, R b, R a, R *ps) {
+__device__ __forceinline__ R pml(R d, bool in, R b, R a, R q, R *ps) {
     if (!in) return d;
-    const R v = b * *ps + a * d;
+    const R v = b * q + a * d;
     *ps = v;
     return d + v;
 }
@@ -70,19 +70,23 @@ __global__ void __launch_bounds__(kHoX *kHoY) k_h_ho(const StepParams<R> p, cons
         const long long idx = (long long)k * plane + (long long)j * pitch + i;
         const bool zin = slab_half(k, nz, npml) >= 0;
         const R bz = zin ? ld(p.az.b_h + k) : R(0), az_ = zin ? ld(p.az.a_h + k) : R(0);
+        R q0 = 0, q1 = 0, q2 = 0, q3 = 0, q4 = 0, q5 = 0;
+        if (yin) { q0 = P[idx]; q5 = P[5 * vol + idx]; }
+        if (zin) { q1 = P[1 * vol + idx]; q2 = P[2 * vol + idx]; }
+        if (xin) { q3 = P[3 * vol + idx]; q4 = P[4 * vol + idx]; }
         if (j < ny && k < nz) {            // Hx at (i, j+1/2, k+1/2)
-            const R a = pml(d_half(Ez, idx, pitch, j, ny, w.wyh), yin, by, ay_, P + idx);
-            const R b = pml(d_half(Ey, idx, plane, k, nz, w.wzh), zin, bz, az_, P + vol + idx);
+            const R a = pml(d_half(Ez, idx, pitch, j, ny, w.wyh), yin, by, ay_, q0, P + idx);
+            const R b = pml(d_half(Ey, idx, plane, k, nz, w.wzh), zin, bz, az_, q1, P + vol + idx);
             Hx[idx] -= cH * (a - b);
         }
         if (i < nx && k < nz) {            // Hy at (i+1/2, j, k+1/2)
-            const R a = pml(d_half(Ex, idx, plane, k, nz, w.wzh), zin, bz, az_, P + 2 * vol + idx);
-            const R b = pml(d_half(Ez, idx, 1LL, i, nx, w.wxh), xin, bx, ax_, P + 3 * vol + idx);
+            const R a = pml(d_half(Ex, idx, plane, k, nz, w.wzh), zin, bz, az_, q2, P + 2 * vol + idx);
+            const R b = pml(d_half(Ez, idx, 1LL, i, nx, w.wxh), xin, bx, ax_, q3, P + 3 * vol + idx);
             Hy[idx] -= cH * (a - b);
         }
         if (i < nx && j < ny) {            // Hz at (i+1/2, j+1/2, k)
-            const R a = pml(d_half(Ey, idx, 1LL, i, nx, w.wxh), xin, bx, ax_, P + 4 * vol + idx);
-            const R b = pml(d_half(Ex, idx, pitch, j, ny, w.wyh), yin, by, ay_, P + 5 * vol + idx);
+            const R a = pml(d_half(Ey, idx, 1LL, i, nx, w.wxh), xin, bx, ax_, q4, P + 4 * vol + idx);
+            const R b = pml(d_half(Ex, idx, pitch, j, ny, w.wyh), yin, by, ay_, q5, P + 5 * vol + idx);
             Hz[idx] -= cH * (a - b);
         }
     }
@@ -114,19 +118,23 @@ __global__ void __launch_bounds__(kHoX *kHoY) k_e_ho(const StepParams<R> p, cons
         const bool zin = slab_node(k, nz, npml) >= 0;
         const R bz = zin ? ld(p.az.b_n + k) : R(0), az_ = zin ? ld(p.az.a_n + k) : R(0);
         const bool kz = (k >= 1 && k < nz);
+        R q0 = 0, q1 = 0, q2 = 0, q3 = 0, q4 = 0, q5 = 0;
+        if (yin) { q0 = P[6 * vol + idx]; q5 = P[11 * vol + idx]; }
+        if (zin) { q1 = P[7 * vol + idx]; q2 = P[8 * vol + idx]; }
+        if (xin) { q3 = P[9 * vol + idx]; q4 = P[10 * vol + idx]; }
         if (i < nx && jy && kz) {          // Ex at (i+1/2, j, k)
-            const R a = pml(d_node(Hz, idx, pitch, j, ny, w.wyn), yin, by, ay_, P + 6 * vol + idx);
-            const R b = pml(d_node(Hy, idx, plane, k, nz, w.wzn), zin, bz, az_, P + 7 * vol + idx);
+            const R a = pml(d_node(Hz, idx, pitch, j, ny, w.wyn), yin, by, ay_, q0, P + 6 * vol + idx);
+            const R b = pml(d_node(Hy, idx, plane, k, nz, w.wzn), zin, bz, az_, q1, P + 7 * vol + idx);
             En[idx] = ld(Eo + idx) + ld(p.cE + idx) * (a - b);
         }
         if (j < ny && ix && kz) {          // Ey at (i, j+1/2, k)
-            const R a = pml(d_node(Hx, idx, plane, k, nz, w.wzn), zin, bz, az_, P + 8 * vol + idx);
-            const R b = pml(d_node(Hz, idx, 1LL, i, nx, w.wxn), xin, bx, ax_, P + 9 * vol + idx);
+            const R a = pml(d_node(Hx, idx, plane, k, nz, w.wzn), zin, bz, az_, q2, P + 8 * vol + idx);
+            const R b = pml(d_node(Hz, idx, 1LL, i, nx, w.wxn), xin, bx, ax_, q3, P + 9 * vol + idx);
             En[vol + idx] = ld(Eo + vol + idx) + ld(p.cE + vol + idx) * (a - b);
         }
         if (k < nz && ix && jy) {          // Ez at (i, j, k+1/2)
-            const R a = pml(d_node(Hy, idx, 1LL, i, nx, w.wxn), xin, bx, ax_, P + 10 * vol + idx);
-            const R b = pml(d_node(Hx, idx, pitch, j, ny, w.wyn), yin, by, ay_, P + 11 * vol + idx);
+            const R a = pml(d_node(Hy, idx, 1LL, i, nx, w.wxn), xin, bx, ax_, q4, P + 10 * vol + idx);
+            const R b = pml(d_node(Hx, idx, pitch, j, ny, w.wyn), yin, by, ay_, q5, P + 11 * vol + idx);
             En[2 * vol + idx] = ld(Eo + 2 * vol + idx) + ld(p.cE + 2 * vol + idx) * (a - b);
         }
     }
@@ -170,6 +178,13 @@ __device__ __forceinline__ const float *at(const float *b, unsigned o) {
 }
 __device__ __forceinline__ float2 f2g(const float *b, unsigned o) { return f2g(at(b, o)); }
 __device__ __forceinline__ float2 f2w(const float *b, unsigned o) { return f2w(at(b, o)); }
+// E^n in the E update, read once and by one thread: past L1, which keeps the rows of H that neighbours read again
+// (512 steps of 128 x 128 x 96: 18.2 -> 17.3 ms)
+__device__ __forceinline__ float2 f2e(const float *b, unsigned o) {
+    float2 r;
+    asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "l"(at(b, o)));
+    return r;
+}
 __device__ __forceinline__ float f1g(const float *b, unsigned o) { return __ldg(at(b, o)); }
 __device__ __forceinline__ float f1w(const float *b, unsigned o) { return *at(b, o); }
 __device__ __forceinline__ void f2s(float *b, unsigned o, float2 v) { f2s(const_cast<float *>(at(b, o)), v); }
@@ -183,16 +198,18 @@ __device__ __forceinline__ float2 dx5(const float4 &w0, const float4 &w1, float 
                                       float f4) {
     return make_float2(w0.x * f0 + w0.y * f1 + w0.z * f2 + w0.w * f3, w1.x * f1 + w1.y * f2 + w1.z * f3 + w1.w * f4);
 }
-__device__ __forceinline__ void pml2(float2 &d, bool in, float b, float a, float *ps, unsigned o) {
+// d with its CPML memory v.  The six entries of a plane are loaded together (H: with the plane's fields; E: after
+// its differences, which leaves the registers of the fields for them).  Loaded one by one, each after the store of
+// the one before it (same array, so the compiler keeps their order), a thread on a slab waited for L2 up to six
+// times per plane: 512 steps of 128 x 128 x 96, 25.6 -> 18.2 ms.
+__device__ __forceinline__ void pml2(float2 &d, bool in, float b, float a, float2 v, float *ps, unsigned o) {
     if (!in) return;
-    float2 v = f2w(ps, o);
     v.x = b * v.x + a * d.x; v.y = b * v.y + a * d.y;
     f2s(ps, o, v);
     d.x += v.x; d.y += v.y;
 }
-__device__ __forceinline__ void pml2x(float2 &d, bool in0, bool in1, float2 b, float2 a, float *ps, unsigned o) {
-    if (!in0 && !in1) return;
-    float2 v = f2w(ps, o);
+__device__ __forceinline__ void pml2x(float2 &d, bool in, float2 b, float2 a, float2 v, float *ps, unsigned o) {
+    if (!in) return;
     v.x = b.x * v.x + a.x * d.x; v.y = b.y * v.y + a.y * d.y;
     f2s(ps, o, v);
     d.x += v.x; d.y += v.y;
@@ -234,7 +251,7 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
     const unsigned im = (i > 0) ? -4 : 0;
     const unsigned jm = (j > 0) ? -4 * pitch : 0, jp = 4 * pitch, jp2 = (j + 2 <= ny) ? 8 * pitch : 4 * (ny - j) * pitch;
     const float4 wx0 = f4g(w.wxh + 4 * i), wx1 = f4g(w.wxh + 4 * (i + 1)), wy = f4g(w.wyh + 4 * j);
-    const bool xs0 = slab_half(i, nx, npml) >= 0, xs1 = slab_half(i + 1, nx, npml) >= 0;
+    const bool xs = slab_half(i, nx, npml) >= 0 || slab_half(i + 1, nx, npml) >= 0;
     const bool ys = slab_half(j, ny, npml) >= 0;
     const float2 bx = make_float2(__ldg(p.lx.b_h + i), __ldg(p.lx.b_h + i + 1));
     const float2 ax = make_float2(__ldg(p.lx.a_h + i), __ldg(p.lx.a_h + i + 1));
@@ -259,18 +276,22 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
         const float2 exm = f2g(Ex, o + jm), exp1 = f2g(Ex, o + jp), exp2 = f2g(Ex, o + jp2);
         const float2 ezm2 = f2g(Ez, o + jm), ezp1 = f2g(Ez, o + jp), ezp2 = f2g(Ez, o + jp2);
         float2 hx = f2w(H, o), hy = f2w(H + vol, o), hz = f2w(H + 2 * vol, o);
+        const bool zs = slab_half(k, nz, npml) >= 0;
+        float2 q0 = {}, q1 = {}, q2 = {}, q3 = {}, q4 = {}, q5 = {};
+        if (ys) { q0 = f2w(P, o); q5 = f2w(P + 5 * vol, o); }
+        if (zs) { q1 = f2w(P + vol, o); q2 = f2w(P + 2 * vol, o); }
+        if (xs) { q3 = f2w(P + 3 * vol, o); q4 = f2w(P + 4 * vol, o); }
         float2 dEz_dy = dot4(wy, ezm2, ez01, ezp1, ezp2), dEy_dz = dot4(wz, ya, yb, yc, yd);
         float2 dEx_dz = dot4(wz, xa, xb, xc, xd), dEz_dx = dx5(wx0, wx1, ezm, ez01.x, ez01.y, ez23.x, ez23.y);
         float2 dEy_dx = dx5(wx0, wx1, eym, yb.x, yb.y, ey23.x, ey23.y), dEx_dy = dot4(wy, exm, xb, exp1, exp2);
-        const bool zs = slab_half(k, nz, npml) >= 0;
-        if (ys || zs || xs0 || xs1) {
+        if (ys || zs || xs) {
             const float bz = __ldg(p.lz.b_h + k), az = __ldg(p.lz.a_h + k);
-            pml2(dEz_dy, ys, by, ay, P, o);
-            pml2(dEy_dz, zs, bz, az, P + vol, o);
-            pml2(dEx_dz, zs, bz, az, P + 2 * vol, o);
-            pml2x(dEz_dx, xs0, xs1, bx, ax, P + 3 * vol, o);
-            pml2x(dEy_dx, xs0, xs1, bx, ax, P + 4 * vol, o);
-            pml2(dEx_dy, ys, by, ay, P + 5 * vol, o);
+            pml2(dEz_dy, ys, by, ay, q0, P, o);
+            pml2(dEy_dz, zs, bz, az, q1, P + vol, o);
+            pml2(dEx_dz, zs, bz, az, q2, P + 2 * vol, o);
+            pml2x(dEz_dx, xs, bx, ax, q3, P + 3 * vol, o);
+            pml2x(dEy_dx, xs, bx, ax, q4, P + 4 * vol, o);
+            pml2(dEx_dy, ys, by, ay, q5, P + 5 * vol, o);
         }
         hx.x -= cH * (dEz_dy.x - dEy_dz.x); hx.y -= cH * (dEz_dy.y - dEy_dz.y);
         hy.x -= cH * (dEx_dz.x - dEz_dx.x); hy.y -= cH * (dEx_dz.y - dEz_dx.y);
@@ -283,12 +304,13 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
     }
 }
 
-template <int KZ, int MINB>
+template <int KZ, int MINB, bool FAR>
 __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, const HoTab<float> w, const int jstep,
                                                      const unsigned S, const unsigned mS) {
     const int i = (blockIdx.x * 32 + threadIdx.x) * 2;
     const int j = blockIdx.y * 4 + threadIdx.y;
-    const int zb = (int)div_by(blockIdx.z, mS), s = (int)(blockIdx.z - zb * S), k0 = zb * KZ;
+    const int zb = (int)div_by(blockIdx.z, mS), s = (int)(blockIdx.z - zb * S);
+    const int k0 = (FAR ? (p.nz + KZ - 1) / KZ - 1 - zb : zb) * KZ;   // downwards where FAR (kFarBytes)
     if (i >= p.nx || j >= p.ny) return;
     const int k1 = min(k0 + KZ, p.nz);
     pdl_wait();
@@ -308,7 +330,7 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
     const unsigned im2 = (i >= 2) ? -8 : -4 * i;
     const unsigned jm2 = (j >= 2) ? -8 * pitch : -4 * j * pitch, jm1 = (j >= 1) ? -4 * pitch : 0, jp = 4 * pitch;
     const float4 wx0 = f4g(w.wxn + 4 * i), wx1 = f4g(w.wxn + 4 * (i + 1)), wy = f4g(w.wyn + 4 * j);
-    const bool xs0 = slab_node(i, nx, npml) >= 0, xs1 = slab_node(i + 1, nx, npml) >= 0;
+    const bool xs = slab_node(i, nx, npml) >= 0 || slab_node(i + 1, nx, npml) >= 0;
     const bool ys = slab_node(j, ny, npml) >= 0;
     const float2 bx = make_float2(__ldg(p.lx.b_n + i), __ldg(p.lx.b_n + i + 1));
     const float2 ax = make_float2(__ldg(p.lx.a_n + i), __ldg(p.lx.a_n + i + 1));
@@ -333,22 +355,26 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
         // y neighbours of Hx, Hz (plane k): rows j-2, j-1, j+1
         const float2 hxm2 = f2w(Hx, o + jm2), hxm1 = f2w(Hx, o + jm1), hxp1 = f2w(Hx, o + jp);
         const float2 hzm2 = f2w(Hz, o + jm2), hzm1 = f2w(Hz, o + jm1), hzp1 = f2w(Hz, o + jp);
-        const float2 e0 = f2g(Eo, o), e1 = f2g(Eo + vol, o), e2 = f2g(Eo + 2 * vol, o);
+        const float2 e0 = f2e(Eo, o), e1 = f2e(Eo + vol, o), e2 = f2e(Eo + 2 * vol, o);
         const float2 c0 = f2g(cE, o), c1 = f2g(cE + vol, o), c2 = f2g(cE + 2 * vol, o);
+        const bool zs = slab_node(k, nz, npml) >= 0;
         float2 dHz_dy = dot4(wy, hzm2, hzm1, hz01, hzp1), dHy_dz = dot4(wz, ya, yb, yc, yd);
         float2 dHx_dz = dot4(wz, xa, xb, xc, xd);
         float2 dHz_dx = dx5(wx0, wx1, hzm.x, hzm.y, hz01.x, hz01.y, hz2);
         float2 dHy_dx = dx5(wx0, wx1, hym.x, hym.y, yc.x, yc.y, hy2);
         float2 dHx_dy = dot4(wy, hxm2, hxm1, xc, hxp1);
-        const bool zs = slab_node(k, nz, npml) >= 0;
-        if (ys || zs || xs0 || xs1) {
+        if (ys || zs || xs) {
+            float2 q0 = {}, q1 = {}, q2 = {}, q3 = {}, q4 = {}, q5 = {};
+            if (ys) { q0 = f2w(P, o); q5 = f2w(P + 5 * vol, o); }
+            if (zs) { q1 = f2w(P + vol, o); q2 = f2w(P + 2 * vol, o); }
+            if (xs) { q3 = f2w(P + 3 * vol, o); q4 = f2w(P + 4 * vol, o); }
             const float bz = __ldg(p.lz.b_n + k), az = __ldg(p.lz.a_n + k);
-            pml2(dHz_dy, ys, by, ay, P, o);
-            pml2(dHy_dz, zs, bz, az, P + vol, o);
-            pml2(dHx_dz, zs, bz, az, P + 2 * vol, o);
-            pml2x(dHz_dx, xs0, xs1, bx, ax, P + 3 * vol, o);
-            pml2x(dHy_dx, xs0, xs1, bx, ax, P + 4 * vol, o);
-            pml2(dHx_dy, ys, by, ay, P + 5 * vol, o);
+            pml2(dHz_dy, ys, by, ay, q0, P, o);
+            pml2(dHy_dz, zs, bz, az, q1, P + vol, o);
+            pml2(dHx_dz, zs, bz, az, q2, P + 2 * vol, o);
+            pml2x(dHz_dx, xs, bx, ax, q3, P + 3 * vol, o);
+            pml2x(dHy_dx, xs, bx, ax, q4, P + 4 * vol, o);
+            pml2(dHx_dy, ys, by, ay, q5, P + 5 * vol, o);
         }
         float2 ex = make_float2(e0.x + c0.x * (dHz_dy.x - dHy_dz.x), e0.y + c0.y * (dHz_dy.y - dHy_dz.y));
         float2 ey = make_float2(e1.x + c1.x * (dHx_dz.x - dHz_dx.x), e1.y + c1.y * (dHx_dz.y - dHz_dx.y));
@@ -374,7 +400,8 @@ void go_ho4k(const StepParams<float> &p, const HoTab<float> &w, int S, int jstep
     const dim3 grid((unsigned)((p.nx / 2 + 31) / 32), (unsigned)((p.ny + 3) / 4), (unsigned)(((p.nz + KZ - 1) / KZ) * S));
     const unsigned mS = div_magic((unsigned)S);
     if (h) launch_pdl(k_h_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS);
-    else launch_pdl(k_e_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS);
+    else if (far_fields(p.vol, S)) launch_pdl(k_e_ho4<KZ, MB, true>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS);
+    else launch_pdl(k_e_ho4<KZ, MB, false>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS);
 }
 template <int MB>
 void go_ho4(const StepParams<float> &p, const HoTab<float> &w, int S, int jstep, cudaStream_t st, bool h, int kz) {

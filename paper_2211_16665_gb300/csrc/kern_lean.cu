@@ -38,17 +38,6 @@ namespace {
 
 constexpr int kLeanX = 32, kLeanRows = 4;
 
-// Order of the E blocks and eviction of H by the bytes of a step's fields (E^n, E^{n+1}, H of every source, dt/eps).
-// Above kFarBytes they do not stay in the 126 MB L2 from one kernel to the next, and with both kernels walking z
-// upwards each found the planes it starts with evicted by those the other one ended with.  There the E blocks walk z
-// downwards, so each kernel starts with the planes that the one before it touched last, and H is stored with
-// evict_last, which keeps H rather than the CPML memory and the E^n that are not read again soon.  Below it the
-// order does not matter (the fields stay in L2) and the policy costs more than it gives.
-// Forward runs of 256 steps, upwards / downwards with the policy: 77 MB (128 x 128 x 96) 6.80 / 6.95 ms, 103 MB
-// (148 x 148 x 96) 10.5 / 10.4, 133 MB 13.5 / 12.6, 166 MB 16.2 / 14.5, 250 MB (four sources of 116^3) 31.3 / 28.8,
-// 700 MB (two of 256 x 256 x 128) 70.0 / 68.4 (downwards alone 68.7).
-constexpr long long kFarBytes = 90LL << 20;
-
 template <int W> struct Vec { float v[W]; };
 template <int W> __device__ __forceinline__ Vec<W> ldc(const float *p) {
     Vec<W> r;
@@ -630,7 +619,7 @@ void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool
     const int nv = (p.nx + W - 1) / W;
     const dim3 grid((nv + kLeanX - 1) / kLeanX, (p.ny + kLeanRows - 1) / kLeanRows, ((p.nz + KZ - 1) / KZ) * S);
     const unsigned mS = div_magic((unsigned)S);
-    const bool far = 12LL * p.vol * (3 * S + 1) > kFarBytes;
+    const bool far = far_fields(p.vol, S);
     if (h && far) launch_pdl(k_h_lean<W, KZ, MB, true>, grid, block, st, p, jstep, (unsigned)S, mS);
     else if (h) launch_pdl(k_h_lean<W, KZ, MB, false>, grid, block, st, p, jstep, (unsigned)S, mS);
     else if (far) launch_pdl(k_e_lean<W, KZ, MB, true>, grid, block, st, p, jstep, (unsigned)S, mS);

@@ -35,3 +35,21 @@ def test_far_batch_equals_single_runs(nx, ny, nz, npml, kz, w):
         assert torch.equal(d[s], d1[0]) and torch.equal(E[s], E1[0])
     eng.check()
     eng.close()
+
+
+@pytest.mark.parametrize("kz", [2, 4, 8])
+def test_far_batch_equals_single_runs_fourth_order(kz):
+    from paper_2211_16665_gb300.engine import Engine
+    wl = W.small_box(n_core=84, n_core_y=81, n_core_z=79, npml=10, n_freq=2, nt=32, n_rec=5)
+    x, z = wl.src.x[0], wl.src.z[0]
+    src = W.Points.make([[x, 0.0, z], [x - 40.0, 90.0, z + 30.0], [x + 60.0, -50.0, z]], [0, 1, 2])
+    eng = Engine.from_workload(wl, max_src=3, autotune=False, order=4)
+    eng.set_launch(kz_h=kz, mb_h=6, lean_h=2, kz_e=kz, mb_e=6, lean_e=2, block=16, flush_mode=1)
+    rho = eng.model_tensor(wl.rho_true)
+    d, E = eng.fwd_model(rho, src, wl.rec, keep_volume=True)
+    assert d.abs().max() > 0
+    for s in range(3):
+        d1, E1 = eng.fwd_model(rho, src.subset([s]), wl.rec, keep_volume=True)
+        assert torch.equal(d[s], d1[0]) and torch.equal(E[s], E1[0])
+    eng.check()
+    eng.close()
