@@ -9,15 +9,19 @@
 //  * the threads of a plane take the cells of the x slabs first and the others after them, so a warp either
 //    needs the x recursion in every lane or not at all (68 cells with 20 of them in the slabs put slab lanes
 //    into every warp of a row-by-row order).  Rows and planes decide on the y and z slabs.
-// 68^3, npml 10: H 28.7 and E 26.6 us per launch with the general kernels (64 % and 58 % of the FP64 pipe's
-// issue slots), 15.0 and 17.7 us with these.
+// The rest is latency: a plane's loads, its CPML memory among them, are issued together (after the stores of the
+// plane's other slabs they came one L2 latency later each), and blocks have 128 threads, so that 4, 6 or 8 of them
+// per SM leave the registers for that.
+// 68^3, npml 10, 1500 steps with volumes: 89.0 ms with the general kernels (H 28.7 and E 26.6 us per launch, 64 % and
+// 58 % of the FP64 pipe's issue slots), 58.3 ms with the fewer operations, 56.7 with the loads together, 53.2 with
+// blocks of 128 too (55.3 with these alone).
 #include "csem_internal.cuh"
 
 namespace csem {
 
 namespace {
 
-constexpr int kB64 = 256;
+constexpr int kB64 = 128;
 
 // The cell (i, j) of thread t of a plane: the x slabs' cells (2 npml per row), padded to whole warps, then the others.
 struct Cell { int i, j; };
@@ -64,26 +68,27 @@ __global__ void __launch_bounds__(kB64, MINB) k_h64(const StepParams<double> p, 
         const double zx = __ldg(Ez + idx + 1) - ezc, yx = __ldg(Ey + idx + 1) - eyc, xy = __ldg(Ex + idx + pitch) - exc;
         const int sz = slab_half(k, nz, npml);
         const double cz = __ldg(p.az.c_h + k);
+        double *qy = psy + (k * np2 + sy) * pitch + i, *qz = psz + (sz * p.NY + j) * pitch + i, *qx = psx + (k * p.NY + j) * np2 + sx;
+        double y0 = 0, y1 = 0, z0 = 0, z1 = 0, x0 = 0, x1 = 0, bz = 0, gz = 0;
+        if (sy >= 0) { y0 = qy[0]; y1 = qy[p.sy]; }
+        if (sz >= 0) { z0 = qz[0]; z1 = qz[p.sz]; bz = __ldg(p.az.b_h + k); gz = __ldg(p.az.g_h + k); }
+        if (sx >= 0) { x0 = qx[0]; x1 = qx[p.sx]; }
         double hx = fma(cz, yz, fma(-cy, zy, H[idx]));
         double hy = fma(cx, zx, fma(-cz, xz, H[vol + idx]));
         double hz = fma(cy, xy, fma(-cx, yx, H[2 * vol + idx]));
         if (sy >= 0) {
-            double *q = psy + (k * np2 + sy) * pitch + i;
-            const double a = fma(gy, zy, by * q[0]), b = fma(gy, xy, by * q[p.sy]);
-            q[0] = a; q[p.sy] = b;
+            const double a = fma(gy, zy, by * y0), b = fma(gy, xy, by * y1);
+            qy[0] = a; qy[p.sy] = b;
             hx -= a; hz += b;
         }
         if (sz >= 0) {
-            const double bz = __ldg(p.az.b_h + k), gz = __ldg(p.az.g_h + k);
-            double *q = psz + (sz * p.NY + j) * pitch + i;
-            const double a = fma(gz, yz, bz * q[0]), b = fma(gz, xz, bz * q[p.sz]);
-            q[0] = a; q[p.sz] = b;
+            const double a = fma(gz, yz, bz * z0), b = fma(gz, xz, bz * z1);
+            qz[0] = a; qz[p.sz] = b;
             hx += a; hy -= b;
         }
         if (sx >= 0) {
-            double *q = psx + (k * p.NY + j) * np2 + sx;
-            const double a = fma(gx, zx, bx * q[0]), b = fma(gx, yx, bx * q[p.sx]);
-            q[0] = a; q[p.sx] = b;
+            const double a = fma(gx, zx, bx * x0), b = fma(gx, yx, bx * x1);
+            qx[0] = a; qx[p.sx] = b;
             hy += a; hz -= b;
         }
         H[idx] = hx; H[vol + idx] = hy; H[2 * vol + idx] = hz;
@@ -124,28 +129,31 @@ __global__ void __launch_bounds__(kB64, MINB) k_e64(const StepParams<double> p, 
         const double zx = hzc - Hz[idx - im], yx = hyc - Hy[idx - im], xy = hxc - Hx[idx - jm];
         const int sz = slab_node(k, nz, npml);
         const double iz = __ldg(p.az.ih_n + k);
+        double *qy = psy + (k * np2 + sy) * pitch + i, *qz = psz + (sz * p.NY + j) * pitch + i, *qx = psx + (k * p.NY + j) * np2 + sx;
+        double y0 = 0, y1 = 0, z0 = 0, z1 = 0, x0 = 0, x1 = 0, bz = 0, gz = 0;
+        if (sy >= 0) { y0 = qy[0]; y1 = qy[p.sy]; }
+        if (sz >= 0) { z0 = qz[0]; z1 = qz[p.sz]; bz = __ldg(p.az.b_n + k); gz = __ldg(p.az.g_n + k); }
+        if (sx >= 0) { x0 = qx[0]; x1 = qx[p.sx]; }
+        const double e0 = __ldg(Eo + idx), e1 = __ldg(Eo + vol + idx), e2 = __ldg(Eo + 2 * vol + idx);
+        const double c0 = __ldg(p.cE + idx), c1 = __ldg(p.cE + vol + idx), c2 = __ldg(p.cE + 2 * vol + idx);
         double tx = fma(-iz, yz, iy * zy), ty = fma(-ix, zx, iz * xz), tz = fma(-iy, xy, ix * yx);
         const bool zin = k >= 1;
         if (sy >= 0) {
-            double *q = psy + (k * np2 + sy) * pitch + i;
-            if (zin) { const double a = fma(gy, zy, by * q[0]); q[0] = a; tx += a; }
-            if (xin) { const double b = fma(gy, xy, by * q[p.sy]); q[p.sy] = b; tz -= b; }
+            if (zin) { const double a = fma(gy, zy, by * y0); qy[0] = a; tx += a; }
+            if (xin) { const double b = fma(gy, xy, by * y1); qy[p.sy] = b; tz -= b; }
         }
         if (sz >= 0) {
-            const double bz = __ldg(p.az.b_n + k), gz = __ldg(p.az.g_n + k);
-            double *q = psz + (sz * p.NY + j) * pitch + i;
-            if (yin) { const double a = fma(gz, yz, bz * q[0]); q[0] = a; tx -= a; }
-            if (xin) { const double b = fma(gz, xz, bz * q[p.sz]); q[p.sz] = b; ty += b; }
+            if (yin) { const double a = fma(gz, yz, bz * z0); qz[0] = a; tx -= a; }
+            if (xin) { const double b = fma(gz, xz, bz * z1); qz[p.sz] = b; ty += b; }
         }
         if (sx >= 0) {
-            double *q = psx + (k * p.NY + j) * np2 + sx;
-            if (zin) { const double a = fma(gx, zx, bx * q[0]); q[0] = a; ty -= a; }
-            if (yin) { const double b = fma(gx, yx, bx * q[p.sx]); q[p.sx] = b; tz += b; }
+            if (zin) { const double a = fma(gx, zx, bx * x0); qx[0] = a; ty -= a; }
+            if (yin) { const double b = fma(gx, yx, bx * x1); qx[p.sx] = b; tz += b; }
         }
         // tangential E on the outer faces keeps its zero
-        if (yin && zin) En[idx] = fma(__ldg(p.cE + idx), tx, __ldg(Eo + idx));
-        if (xin && zin) En[vol + idx] = fma(__ldg(p.cE + vol + idx), ty, __ldg(Eo + vol + idx));
-        if (xin && yin) En[2 * vol + idx] = fma(__ldg(p.cE + 2 * vol + idx), tz, __ldg(Eo + 2 * vol + idx));
+        if (yin && zin) En[idx] = fma(c0, tx, e0);
+        if (xin && zin) En[vol + idx] = fma(c1, ty, e1);
+        if (xin && yin) En[2 * vol + idx] = fma(c2, tz, e2);
         hxm = hxc;
         hym = hyc;
     }
