@@ -286,8 +286,7 @@ cudaError_t launch_step_ws(const StepParams<float> &p, int S, int jstep, cudaStr
 bool ws_supported(int by, int mb, int kz);
 // FP64 H / E kernels (kern_f64.cu), kz in {1,2,4,8}, mb in {4,6,8}
 cudaError_t launch_field64(const StepParams<double> &p, int S, int jstep, cudaStream_t st, bool h, int kz, int mb);
-// FP32 H / E kernels with four cells per thread (kern_vec.cu), kz in {1,2,4,8}, mb in {4,6}
-// lean FP32 H / E kernels (kern_lean.cu), nx % 4 == 0, w (cells per thread) in {1,2}, kz in {1,2,4},
+// lean FP32 H / E kernels (kern_lean.cu), any nx, w (cells per thread) in {1,2}, kz in {1,2,4},
 // mb (resident 128-thread blocks per SM) in {6,8} for w = 1 and {4,6,8} for w = 2
 cudaError_t launch_field_lean(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int w, int kz,
                               int mb);
@@ -300,6 +299,7 @@ bool wave_supported(const StepParams<float> &p, int kz, int mb);
 cudaError_t launch_mask_coef(const StepParams<float> &p, const float *cE, float *cEm, cudaStream_t st);
 // p.inc for the steps jstep in [0, nsteps) after *p.step (zero past nt)
 cudaError_t launch_tap_inc(const StepParams<float> &p, int S, int nsteps, int nt, cudaStream_t st);
+// FP32 H / E kernels with four cells per thread (kern_vec.cu), kz in {1,2,4,8}, mb in {4,6}
 cudaError_t launch_field_vec(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int kz, int mb);
 // FP32 bulk-copy-staged H / E kernels (kern_tma.cu): ty rows per block in {1,2,4}, kz planes per chunk
 cudaError_t launch_field_tma(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int kz, int ty,

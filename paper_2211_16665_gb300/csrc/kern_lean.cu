@@ -31,6 +31,10 @@
 // resident blocks per SM give 128, 85 or 64 registers per thread); blockIdx.z
 // runs over (z block, source) with the source fastest; the planes of the last, partial
 // wave of blocks go to blocks of one plane (big_blocks).
+// What bounds them: DRAM where the fields exceed L2 (two sources of 256 x 256 x 128 move
+// their bytes at the rate of a copy, so only bytes count: see kFarBytes), L2 latency and
+// the partial wave where they fit (128 x 128 x 96: 27 us a step, 24 with big_blocks and
+// E^n past L1), and the launches themselves below about 10^5 cells.
 #include "csem_internal.cuh"
 
 namespace csem {
