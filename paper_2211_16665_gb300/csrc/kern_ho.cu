@@ -5,6 +5,8 @@
 // touched only inside its slabs.  E lives in the same ring of snapshots as in
 // the second-order kernels (E^{n+1} is written to slot n+1 from slot n), and the
 // E kernel applies the source injection of its column's taps.
+#include <algorithm>
+
 #include "csem_ho.cuh"
 
 namespace csem {
@@ -229,12 +231,12 @@ __device__ __forceinline__ float3 ho_taps(const int *__restrict__ tk, const floa
 
 template <int KZ, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, const HoTab<float> w, const int jstep,
-                                                     const unsigned S, const unsigned mS) {
+                                                     const unsigned S, const unsigned mS, const int nbig) {
     const int i = (blockIdx.x * 32 + threadIdx.x) * 2;
     const int j = blockIdx.y * 4 + threadIdx.y;
-    const int zb = (int)div_by(blockIdx.z, mS), s = (int)(blockIdx.z - zb * S), k0 = zb * KZ;
+    const int zb = (int)div_by(blockIdx.z, mS), s = (int)(blockIdx.z - zb * S);
+    const int k0 = zb < nbig ? zb * KZ : nbig * KZ + (zb - nbig), k1 = min(k0 + (zb < nbig ? KZ : 1), p.nz);   // big_blocks
     if (i >= p.nx || j >= p.ny) return;
-    const int k1 = min(k0 + KZ, p.nz);
     pdl_wait();
     const int sl = slot_of(p, *p.step + jstep);
     const int nx = p.nx, ny = p.ny, nz = p.nz, npml = p.npml;
@@ -306,13 +308,14 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
 
 template <int KZ, int MINB, bool FAR>
 __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, const HoTab<float> w, const int jstep,
-                                                     const unsigned S, const unsigned mS) {
+                                                     const unsigned S, const unsigned mS, const int nbig) {
     const int i = (blockIdx.x * 32 + threadIdx.x) * 2;
     const int j = blockIdx.y * 4 + threadIdx.y;
     const int zb = (int)div_by(blockIdx.z, mS), s = (int)(blockIdx.z - zb * S);
-    const int k0 = (FAR ? (p.nz + KZ - 1) / KZ - 1 - zb : zb) * KZ;   // downwards where FAR (kFarBytes)
+    const int at = zb < nbig ? zb * KZ : nbig * KZ + (zb - nbig), len = zb < nbig ? KZ : 1;   // big_blocks
+    const int k0 = FAR ? max(p.nz - at - len, 0) : at;       // downwards where FAR (kFarBytes)
+    const int k1 = FAR ? p.nz - at : min(at + len, p.nz);
     if (i >= p.nx || j >= p.ny) return;
-    const int k1 = min(k0 + KZ, p.nz);
     pdl_wait();
     const int sl = slot_of(p, *p.step + jstep);
     const int nx = p.nx, ny = p.ny, nz = p.nz, npml = p.npml;
@@ -397,11 +400,13 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
 
 template <int KZ, int MB>
 void go_ho4k(const StepParams<float> &p, const HoTab<float> &w, int S, int jstep, cudaStream_t st, bool h) {
-    const dim3 grid((unsigned)((p.nx / 2 + 31) / 32), (unsigned)((p.ny + 3) / 4), (unsigned)(((p.nz + KZ - 1) / KZ) * S));
+    const int gx = (p.nx / 2 + 31) / 32, gy = (p.ny + 3) / 4, nzb = (p.nz + KZ - 1) / KZ;
+    const int nbig = big_blocks(nzb, KZ, gx * gy * S, MB);
+    const dim3 grid(gx, gy, (nbig + std::max(p.nz - nbig * KZ, 0)) * S);
     const unsigned mS = div_magic((unsigned)S);
-    if (h) launch_pdl(k_h_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS);
-    else if (far_fields(p.vol, S)) launch_pdl(k_e_ho4<KZ, MB, true>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS);
-    else launch_pdl(k_e_ho4<KZ, MB, false>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS);
+    if (h) launch_pdl(k_h_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS, nbig);
+    else if (far_fields(p.vol, S)) launch_pdl(k_e_ho4<KZ, MB, true>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS, nbig);
+    else launch_pdl(k_e_ho4<KZ, MB, false>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS, nbig);
 }
 template <int MB>
 void go_ho4(const StepParams<float> &p, const HoTab<float> &w, int S, int jstep, cudaStream_t st, bool h, int kz) {

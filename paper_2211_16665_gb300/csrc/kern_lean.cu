@@ -29,10 +29,11 @@
 // W stays small so that a plane's loaded values fit the register budget.
 // The block is 32 x 4 threads (32 W cells of 4 rows; 128 threads, so 4, 6 or 8
 // resident blocks per SM give 128, 85 or 64 registers per thread); blockIdx.z
-// runs over (z block, source) with the source fastest.
+// runs over (z block, source) with the source fastest; the planes of the last, partial
+// wave of blocks go to blocks of one plane (big_blocks).
 // What bounds them: DRAM where the fields exceed L2 (two sources of 256 x 256 x 128 move
 // their bytes at the rate of a copy, so only bytes count: see kFarBytes), L2 latency and
-// the last, partial wave of blocks where they fit (128 x 128 x 96: 27 us a step, 25 with
+// the partial wave where they fit (128 x 128 x 96: 27 us a step, 24 with big_blocks and
 // E^n past L1), and the launches themselves below about 10^5 cells.
 #include "csem_internal.cuh"
 
@@ -97,40 +98,56 @@ template <int W> __device__ __forceinline__ Vec<W> zv() {
     for (int e = 0; e < W; ++e) r.v[e] = 0.f;
     return r;
 }
-// (a - b) * s
-template <int W> __device__ __forceinline__ Vec<W> dsc(const Vec<W> &a, const Vec<W> &b, float s) {
+// The roundings are spelled out, so that every instance of the kernels (cells and planes per thread, registers, order)
+// gives the same bits: left to itself the compiler fused one product or the other of a sum of two, by instance.
+// a - b
+template <int W> __device__ __forceinline__ Vec<W> dif(const Vec<W> &a, const Vec<W> &b) {
     Vec<W> r;
 #pragma unroll
-    for (int e = 0; e < W; ++e) r.v[e] = (a.v[e] - b.v[e]) * s;
+    for (int e = 0; e < W; ++e) r.v[e] = __fsub_rn(a.v[e], b.v[e]);
     return r;
 }
-template <int W> __device__ __forceinline__ Vec<W> dsc(const Vec<W> &a, const Vec<W> &b, const Vec<W> &s) {
+// a s (shared or per-cell s)
+template <int W> __device__ __forceinline__ Vec<W> mul(const Vec<W> &a, float s) {
     Vec<W> r;
 #pragma unroll
-    for (int e = 0; e < W; ++e) r.v[e] = (a.v[e] - b.v[e]) * s.v[e];
+    for (int e = 0; e < W; ++e) r.v[e] = __fmul_rn(a.v[e], s);
     return r;
 }
-// CPML recursion psi <- b psi + a d, then d += psi (shared or per-cell b, a)
+template <int W> __device__ __forceinline__ Vec<W> mul(const Vec<W> &a, const Vec<W> &s) {
+    Vec<W> r;
+#pragma unroll
+    for (int e = 0; e < W; ++e) r.v[e] = __fmul_rn(a.v[e], s.v[e]);
+    return r;
+}
+// a s + c with one rounding
+template <int W> __device__ __forceinline__ Vec<W> mad(const Vec<W> &a, float s, const Vec<W> &c) {
+    Vec<W> r;
+#pragma unroll
+    for (int e = 0; e < W; ++e) r.v[e] = fmaf(a.v[e], s, c.v[e]);
+    return r;
+}
+template <int W> __device__ __forceinline__ Vec<W> mad(const Vec<W> &a, const Vec<W> &s, const Vec<W> &c) {
+    Vec<W> r;
+#pragma unroll
+    for (int e = 0; e < W; ++e) r.v[e] = fmaf(a.v[e], s.v[e], c.v[e]);
+    return r;
+}
+template <int W> __device__ __forceinline__ Vec<W> neg(const Vec<W> &a) {
+    Vec<W> r;
+#pragma unroll
+    for (int e = 0; e < W; ++e) r.v[e] = -a.v[e];
+    return r;
+}
+// CPML recursion psi <- b psi + a d, then d += psi (shared or per-cell b, a).  b psi is rounded and a d fused to it:
+// the product that does not wait for the field loads goes first (the other way round 256 x 256 x 128 took 1 % longer).
 template <int W> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, float b, float a) {
 #pragma unroll
-    for (int e = 0; e < W; ++e) { ps.v[e] = b * ps.v[e] + a * d.v[e]; d.v[e] += ps.v[e]; }
+    for (int e = 0; e < W; ++e) { ps.v[e] = fmaf(a, d.v[e], __fmul_rn(b, ps.v[e])); d.v[e] = __fadd_rn(d.v[e], ps.v[e]); }
 }
 template <int W> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, const Vec<W> &b, const Vec<W> &a) {
 #pragma unroll
-    for (int e = 0; e < W; ++e) { ps.v[e] = b.v[e] * ps.v[e] + a.v[e] * d.v[e]; d.v[e] += ps.v[e]; }
-}
-// h -= c (u - v)
-template <int W> __device__ __forceinline__ void hsub(Vec<W> &h, float c, const Vec<W> &u, const Vec<W> &v) {
-#pragma unroll
-    for (int e = 0; e < W; ++e) h.v[e] -= c * (u.v[e] - v.v[e]);
-}
-// eo + c (u - v)
-template <int W>
-__device__ __forceinline__ Vec<W> eadv(const Vec<W> &eo, const Vec<W> &c, const Vec<W> &u, const Vec<W> &v) {
-    Vec<W> r;
-#pragma unroll
-    for (int e = 0; e < W; ++e) r.v[e] = eo.v[e] + c.v[e] * (u.v[e] - v.v[e]);
-    return r;
+    for (int e = 0; e < W; ++e) { ps.v[e] = fmaf(a.v[e], d.v[e], __fmul_rn(b.v[e], ps.v[e])); d.v[e] = __fadd_rn(d.v[e], ps.v[e]); }
 }
 // the W cells shifted by one: (prev, a0, .., a_{W-2}) and (a1, .., a_{W-1}, next)
 template <int W> __device__ __forceinline__ Vec<W> down(float prev, const Vec<W> &a) {
@@ -228,22 +245,35 @@ __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float 
     const Vec<W> ezx = up<W>(ezc, ezn), eyx = up<W>(eyc, eyn);   // Ez, Ey at i+1 .. i+W
 
     // Hx at (i, j+1/2, k+1/2)
-    Vec<W> dEz_dy = dsc<W>(ezj, ezc, r.ihy), dEy_dz = dsc<W>(eyk, eyc, ihz);
-    if (YZ && ys) { cpml<W>(q0, dEz_dy, r.by, r.ay); stv<W>(ps, o, q0); }
-    if (YZ && zs) { cpml<W>(q1, dEy_dz, bz, az); stv<W>(ps + vol, o, q1); }
-    hsub<W>(hx, p.cH, dEz_dy, dEy_dz);
+    Vec<W> zy = dif<W>(ezj, ezc), yz = dif<W>(eyk, eyc), c;
+    if constexpr (YZ) {
+        zy = mul<W>(zy, r.ihy); yz = mul<W>(yz, ihz);
+        if (ys) { cpml<W>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
+        if (zs) { cpml<W>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
+        c = dif<W>(zy, yz);
+    } else c = mad<W>(zy, r.ihy, mul<W>(yz, -ihz));
+    hx = mad<W>(c, -p.cH, hx);
     // Hy at (i+1/2, j, k+1/2)
-    Vec<W> dEx_dz = dsc<W>(exk, exc, ihz), dEz_dx = dsc<W>(ezx, ezc, r.ihx);
-    if (YZ && zs) { cpml<W>(q2, dEx_dz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
-    cpml<W>(q3, dEz_dx, r.bx, r.ax);
+    Vec<W> xz = dif<W>(exk, exc), zx = mul<W>(dif<W>(ezx, ezc), r.ihx);
+    if constexpr (YZ) {
+        xz = mul<W>(xz, ihz);
+        if (zs) { cpml<W>(q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
+    }
+    cpml<W>(q3, zx, r.bx, r.ax);
     if (r.xs) stv<W>(px3, xo, q3);
-    hsub<W>(hy, p.cH, dEx_dz, dEz_dx);
+    if constexpr (YZ) c = dif<W>(xz, zx);
+    else c = mad<W>(xz, ihz, neg<W>(zx));
+    hy = mad<W>(c, -p.cH, hy);
     // Hz at (i+1/2, j+1/2, k)
-    Vec<W> dEy_dx = dsc<W>(eyx, eyc, r.ihx), dEx_dy = dsc<W>(exj, exc, r.ihy);
-    cpml<W>(q4, dEy_dx, r.bx, r.ax);
+    Vec<W> yx = mul<W>(dif<W>(eyx, eyc), r.ihx), xy = dif<W>(exj, exc);
+    cpml<W>(q4, yx, r.bx, r.ax);
     if (r.xs) stv<W>(px4, xo, q4);
-    if (YZ && ys) { cpml<W>(q5, dEx_dy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
-    hsub<W>(hz, p.cH, dEy_dx, dEx_dy);
+    if constexpr (YZ) {
+        xy = mul<W>(xy, r.ihy);
+        if (ys) { cpml<W>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
+        c = dif<W>(yx, xy);
+    } else c = mad<W>(xy, -r.ihy, yx);
+    hz = mad<W>(c, -p.cH, hz);
 
     if constexpr (FAR) { stl<W>(H, o, hx); stl<W>(Hy, o, hy); stl<W>(Hz, o, hz); }
     else { stv<W>(H, o, hx); stv<W>(Hy, o, hy); stv<W>(Hz, o, hz); }
@@ -284,15 +314,16 @@ __device__ __forceinline__ void h_tile(const StepParams<float> &p, const int jst
     }
 }
 
-template <int W, int KZ, int MINB, bool FAR>
+template <int W, int KZ, int MINB, bool FAR, bool TAIL>
 __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepParams<float> p, const int jstep, const unsigned S,
-                                                                       const unsigned mS) {
+                                                                       const unsigned mS, const int nbig) {
     const int i = (blockIdx.x * kLeanX + threadIdx.x) * W;
     const int j = blockIdx.y * kLeanRows + threadIdx.y;
     const int zb = (int)div_by(blockIdx.z, mS);   // the source runs fastest: the sources of one
-    const int s = (int)(blockIdx.z - zb * S), k0 = zb * KZ;    // z block follow one another
+    const int s = (int)(blockIdx.z - zb * S);     // z block follow one another
+    const bool one = TAIL && zb >= nbig;          // big_blocks
+    const int k0 = one ? nbig * KZ + (zb - nbig) : zb * KZ, k1 = min(k0 + (one ? 1 : KZ), p.nz);
     if (i >= p.nx || j >= p.ny) return;
-    const int k1 = min(k0 + KZ, p.nz);
     const int plane = (int)p.plane, npml = p.npml;
     const long long vol = p.vol;
     LeanRow<W> r;
@@ -365,22 +396,35 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
     const Vec<W> hzx = down<W>(hzp, hzc), hyx = down<W>(hyp, hyc);   // Hz, Hy at i-1 .. i+W-2
 
     // Ex at (i+1/2, j, k)
-    Vec<W> dHz_dy = dsc<W>(hzc, hzj, r.ihy), dHy_dz = dsc<W>(hyc, hym, ihz);
-    if (YZ && ys) { cpml<W>(q0, dHz_dy, r.by, r.ay); stv<W>(ps, o, q0); }
-    if (YZ && zs) { cpml<W>(q1, dHy_dz, bz, az); stv<W>(ps + vol, o, q1); }
-    Vec<W> e0 = eadv<W>(eo0, c0, dHz_dy, dHy_dz);
+    Vec<W> zy = dif<W>(hzc, hzj), yz = dif<W>(hyc, hym), c;
+    if constexpr (YZ) {
+        zy = mul<W>(zy, r.ihy); yz = mul<W>(yz, ihz);
+        if (ys) { cpml<W>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
+        if (zs) { cpml<W>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
+        c = dif<W>(zy, yz);
+    } else c = mad<W>(zy, r.ihy, mul<W>(yz, -ihz));
+    Vec<W> e0 = mad<W>(c, c0, eo0);
     // Ey at (i, j+1/2, k)
-    Vec<W> dHx_dz = dsc<W>(hxc, hxm, ihz), dHz_dx = dsc<W>(hzc, hzx, r.ihx);
-    if (YZ && zs) { cpml<W>(q2, dHx_dz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
-    cpml<W>(q3, dHz_dx, r.bx, r.ax);
+    Vec<W> xz = dif<W>(hxc, hxm), zx = mul<W>(dif<W>(hzc, hzx), r.ihx);
+    if constexpr (YZ) {
+        xz = mul<W>(xz, ihz);
+        if (zs) { cpml<W>(q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
+    }
+    cpml<W>(q3, zx, r.bx, r.ax);
     if (r.xs) stv<W>(px3, xo, q3);
-    Vec<W> e1 = eadv<W>(eo1, c1, dHx_dz, dHz_dx);
+    if constexpr (YZ) c = dif<W>(xz, zx);
+    else c = mad<W>(xz, ihz, neg<W>(zx));
+    Vec<W> e1 = mad<W>(c, c1, eo1);
     // Ez at (i, j, k+1/2)
-    Vec<W> dHy_dx = dsc<W>(hyc, hyx, r.ihx), dHx_dy = dsc<W>(hxc, hxj, r.ihy);
-    cpml<W>(q4, dHy_dx, r.bx, r.ax);
+    Vec<W> yx = mul<W>(dif<W>(hyc, hyx), r.ihx), xy = dif<W>(hxc, hxj);
+    cpml<W>(q4, yx, r.bx, r.ax);
     if (r.xs) stv<W>(px4, xo, q4);
-    if (YZ && ys) { cpml<W>(q5, dHx_dy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
-    Vec<W> e2 = eadv<W>(eo2, c2, dHy_dx, dHx_dy);
+    if constexpr (YZ) {
+        xy = mul<W>(xy, r.ihy);
+        if (ys) { cpml<W>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
+        c = dif<W>(yx, xy);
+    } else c = mad<W>(xy, -r.ihy, yx);
+    Vec<W> e2 = mad<W>(c, c2, eo2);
 
     if (taps) {
         const int2 *cm = p.colmap + (long long)s * p.colmap_stride + r.j * p.pitch + r.i;
@@ -438,16 +482,20 @@ __device__ __forceinline__ void e_tile(const StepParams<float> &p, const int jst
     }
 }
 
-template <int W, int KZ, int MINB, bool FAR>
+template <int W, int KZ, int MINB, bool FAR, bool TAIL>
 __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepParams<float> p, const int jstep, const unsigned S,
-                                                                       const unsigned mS) {
+                                                                       const unsigned mS, const int nbig) {
     const int i = (blockIdx.x * kLeanX + threadIdx.x) * W;
     const int j = blockIdx.y * kLeanRows + threadIdx.y;
     const int zq = (int)div_by(blockIdx.z, mS);   // the source runs fastest: the sources of one z
     const int s = (int)(blockIdx.z - zq * S);     // block share the dt/eps reads in L2
-    const int k0 = (FAR ? (p.nz + KZ - 1) / KZ - 1 - zq : zq) * KZ;   // downwards where FAR (kFarBytes)
+    int k0 = (FAR ? (p.nz + KZ - 1) / KZ - 1 - zq : zq) * KZ, k1 = min(k0 + KZ, p.nz);   // downwards where FAR (kFarBytes)
+    if constexpr (TAIL) {                         // big_blocks
+        const int at = zq < nbig ? zq * KZ : nbig * KZ + (zq - nbig), len = zq < nbig ? KZ : 1;
+        k0 = FAR ? max(p.nz - at - len, 0) : at;
+        k1 = FAR ? p.nz - at : min(at + len, p.nz);
+    }
     if (i >= p.nx || j >= p.ny) return;
-    const int k1 = min(k0 + KZ, p.nz);
     LeanRow<W> r;
     lean_row<W>(p, p.lx, p.ly, false, i, j, r);
     pdl_wait();
@@ -617,17 +665,24 @@ __global__ void k_mask_coef(const StepParams<float> p, const float *__restrict__
 }
 
 namespace {
-template <int W, int KZ, int MB>
-void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h) {
+template <int W, int KZ, int MB, bool TAIL>
+void lean_launch(const StepParams<float> &p, dim3 grid, int nbig, int S, int jstep, cudaStream_t st, bool h) {
     const dim3 block(kLeanX, kLeanRows);
-    const int nv = (p.nx + W - 1) / W;
-    const dim3 grid((nv + kLeanX - 1) / kLeanX, (p.ny + kLeanRows - 1) / kLeanRows, ((p.nz + KZ - 1) / KZ) * S);
     const unsigned mS = div_magic((unsigned)S);
     const bool far = far_fields(p.vol, S);
-    if (h && far) launch_pdl(k_h_lean<W, KZ, MB, true>, grid, block, st, p, jstep, (unsigned)S, mS);
-    else if (h) launch_pdl(k_h_lean<W, KZ, MB, false>, grid, block, st, p, jstep, (unsigned)S, mS);
-    else if (far) launch_pdl(k_e_lean<W, KZ, MB, true>, grid, block, st, p, jstep, (unsigned)S, mS);
-    else launch_pdl(k_e_lean<W, KZ, MB, false>, grid, block, st, p, jstep, (unsigned)S, mS);
+    if (h && far) launch_pdl(k_h_lean<W, KZ, MB, true, TAIL>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+    else if (h) launch_pdl(k_h_lean<W, KZ, MB, false, TAIL>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+    else if (far) launch_pdl(k_e_lean<W, KZ, MB, true, TAIL>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+    else launch_pdl(k_e_lean<W, KZ, MB, false, TAIL>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+}
+template <int W, int KZ, int MB>
+void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h) {
+    const int nv = (p.nx + W - 1) / W, nzb = (p.nz + KZ - 1) / KZ;
+    const int gx = (nv + kLeanX - 1) / kLeanX, gy = (p.ny + kLeanRows - 1) / kLeanRows;
+    const int nbig = big_blocks(nzb, KZ, gx * gy * S, MB);
+    if constexpr (KZ > 1)
+        if (nbig < nzb) return lean_launch<W, KZ, MB, true>(p, dim3(gx, gy, (nbig + p.nz - nbig * KZ) * S), nbig, S, jstep, st, h);
+    lean_launch<W, KZ, MB, false>(p, dim3(gx, gy, nzb * S), nzb, S, jstep, st, h);
 }
 template <int W, int MB>
 bool lean_kz(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int kz) {
