@@ -98,8 +98,12 @@ template <int W> __device__ __forceinline__ Vec<W> zv() {
     for (int e = 0; e < W; ++e) r.v[e] = 0.f;
     return r;
 }
-// The roundings are spelled out, so that every instance of the kernels (cells and planes per thread, registers, order)
-// gives the same bits: left to itself the compiler fused one product or the other of a sum of two, by instance.
+// The roundings are spelled out.  Left to itself the compiler fuses one product or the other of a sum of two, by
+// instance; a gradient multiplies such a difference by up to 10^4 (the adjoint basis is ill-conditioned), so it then
+// changes with every new instance of a kernel.  Here every instance with the same planes per thread gives the same
+// bits, whatever its cells per thread, blocks per SM, order and size of its z blocks.  Which products are fused follows
+// the kernels that were compiled from the plain expressions, so results are what they were: h_plane and e_plane say
+// where.
 // a - b
 template <int W> __device__ __forceinline__ Vec<W> dif(const Vec<W> &a, const Vec<W> &b) {
     Vec<W> r;
@@ -139,15 +143,25 @@ template <int W> __device__ __forceinline__ Vec<W> neg(const Vec<W> &a) {
     for (int e = 0; e < W; ++e) r.v[e] = -a.v[e];
     return r;
 }
-// CPML recursion psi <- b psi + a d, then d += psi (shared or per-cell b, a).  b psi is rounded and a d fused to it:
-// the product that does not wait for the field loads goes first (the other way round 256 x 256 x 128 took 1 % longer).
+// CPML recursion psi <- b psi + a d, then d += psi (shared or per-cell b, a); b psi is fused to the rounded a d.
+__device__ __forceinline__ void cpml1(float &ps, float &d, float b, float a) {
+    ps = fmaf(b, ps, __fmul_rn(a, d));
+    d = __fadd_rn(d, ps);
+}
 template <int W> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, float b, float a) {
 #pragma unroll
-    for (int e = 0; e < W; ++e) { ps.v[e] = fmaf(a, d.v[e], __fmul_rn(b, ps.v[e])); d.v[e] = __fadd_rn(d.v[e], ps.v[e]); }
+    for (int e = 0; e < W; ++e) cpml1(ps.v[e], d.v[e], b, a);
 }
 template <int W> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, const Vec<W> &b, const Vec<W> &a) {
 #pragma unroll
-    for (int e = 0; e < W; ++e) { ps.v[e] = fmaf(a.v[e], d.v[e], __fmul_rn(b.v[e], ps.v[e])); d.v[e] = __fadd_rn(d.v[e], ps.v[e]); }
+    for (int e = 0; e < W; ++e) cpml1(ps.v[e], d.v[e], b.v[e], a.v[e]);
+}
+// u s - v and v - u s, the product rounded first or (fuse) fused to v
+template <int W> __device__ __forceinline__ Vec<W> mulsub(bool fuse, const Vec<W> &u, float s, const Vec<W> &v) {
+    return fuse ? mad<W>(u, s, neg<W>(v)) : dif<W>(mul<W>(u, s), v);
+}
+template <int W> __device__ __forceinline__ Vec<W> submul(bool fuse, const Vec<W> &v, const Vec<W> &u, float s) {
+    return fuse ? mad<W>(u, -s, v) : dif<W>(v, mul<W>(u, s));
 }
 // the W cells shifted by one: (prev, a0, .., a_{W-2}) and (a1, .., a_{W-1}, next)
 template <int W> __device__ __forceinline__ Vec<W> down(float prev, const Vec<W> &a) {
@@ -212,11 +226,12 @@ __device__ __forceinline__ float3 lean_taps(const int *__restrict__ tk, const fl
 }  // namespace
 
 // One plane k of the H update for the thread's W cells; YZ: the y/z recursion
-// may apply (a block on a y or z slab); FAR: see kFarBytes.  o: byte offset of the cells in a component,
+// may apply (a block on a y or z slab); FAR: see kFarBytes.  Off the slabs the products
+// of a difference are fused, but for those of Hy and Hz in the last plane of a z block of KZ planes (last).  o: byte offset of the cells in a component,
 // xo: of their x-slab entries.  exc, eyc: Ex, Ey of plane k (in), of plane k+1 (out).
 template <int W, bool YZ, bool FAR>
 __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float *__restrict__ E, float *__restrict__ H,
-                                        float *__restrict__ ps, const LeanRow<W> &r, int k, unsigned o, unsigned xo,
+                                        float *__restrict__ ps, const LeanRow<W> &r, int k, bool last, unsigned o, unsigned xo,
                                         Vec<W> &exc, Vec<W> &eyc) {
     const long long vol = p.vol;
     const unsigned plane = 4u * (unsigned)p.plane, pitch = 4u * (unsigned)p.pitch;
@@ -251,7 +266,7 @@ __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float 
         if (ys) { cpml<W>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
         if (zs) { cpml<W>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
         c = dif<W>(zy, yz);
-    } else c = mad<W>(zy, r.ihy, mul<W>(yz, -ihz));
+    } else c = mulsub<W>(true, zy, r.ihy, mul<W>(yz, ihz));
     hx = mad<W>(c, -p.cH, hx);
     // Hy at (i+1/2, j, k+1/2)
     Vec<W> xz = dif<W>(exk, exc), zx = mul<W>(dif<W>(ezx, ezc), r.ihx);
@@ -262,7 +277,7 @@ __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float 
     cpml<W>(q3, zx, r.bx, r.ax);
     if (r.xs) stv<W>(px3, xo, q3);
     if constexpr (YZ) c = dif<W>(xz, zx);
-    else c = mad<W>(xz, ihz, neg<W>(zx));
+    else c = mulsub<W>(!last, xz, ihz, zx);
     hy = mad<W>(c, -p.cH, hy);
     // Hz at (i+1/2, j+1/2, k)
     Vec<W> yx = mul<W>(dif<W>(eyx, eyc), r.ihx), xy = dif<W>(exj, exc);
@@ -272,7 +287,7 @@ __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float 
         xy = mul<W>(xy, r.ihy);
         if (ys) { cpml<W>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
         c = dif<W>(yx, xy);
-    } else c = mad<W>(xy, -r.ihy, yx);
+    } else c = submul<W>(!last, yx, xy, r.ihy);
     hz = mad<W>(c, -p.cH, hz);
 
     if constexpr (FAR) { stl<W>(H, o, hx); stl<W>(Hy, o, hy); stl<W>(Hz, o, hz); }
@@ -309,8 +324,8 @@ __device__ __forceinline__ void h_tile(const StepParams<float> &p, const int jst
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, false>(p, E, H, ps, r, k, o, xo, exc, eyc);
-        else h_plane<W, false, false>(p, E, H, ps, r, k, o, xo, exc, eyc);
+        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, false>(p, E, H, ps, r, k, kk == KZ - 1, o, xo, exc, eyc);
+        else h_plane<W, false, false>(p, E, H, ps, r, k, kk == KZ - 1, o, xo, exc, eyc);
     }
 }
 
@@ -343,8 +358,9 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepPa
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, FAR>(p, E, H, ps, r, k, o, xo, exc, eyc);
-        else h_plane<W, false, FAR>(p, E, H, ps, r, k, o, xo, exc, eyc);
+        const bool last = TAIL ? (k & (KZ - 1)) == KZ - 1 : kk == KZ - 1;   // z blocks start at multiples of KZ without big_blocks
+        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, FAR>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
+        else h_plane<W, false, FAR>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
     }
 }
 
@@ -368,8 +384,8 @@ template <bool CG> __device__ __forceinline__ float ldh1(const float *b, unsigne
 template <int W, bool YZ, bool CG>
 __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float *__restrict__ Eo, float *__restrict__ En,
                                         const float *__restrict__ H, float *__restrict__ ps, const LeanRow<W> &r, int s,
-                                        int S, int jstep, int k, unsigned o, unsigned xo, unsigned oj, unsigned oi,
-                                        bool taps, Vec<W> &hxm, Vec<W> &hym) {
+                                        int S, int jstep, int k, bool last, unsigned o, unsigned xo, unsigned oj,
+                                        unsigned oi, bool taps, Vec<W> &hxm, Vec<W> &hym) {
     const long long vol = p.vol;
     const int npml = p.npml;
     const float *__restrict__ cE = p.cEm;
@@ -402,7 +418,7 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
         if (ys) { cpml<W>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
         if (zs) { cpml<W>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
         c = dif<W>(zy, yz);
-    } else c = mad<W>(zy, r.ihy, mul<W>(yz, -ihz));
+    } else c = mulsub<W>(true, zy, r.ihy, mul<W>(yz, ihz));
     Vec<W> e0 = mad<W>(c, c0, eo0);
     // Ey at (i, j+1/2, k)
     Vec<W> xz = dif<W>(hxc, hxm), zx = mul<W>(dif<W>(hzc, hzx), r.ihx);
@@ -413,7 +429,7 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
     cpml<W>(q3, zx, r.bx, r.ax);
     if (r.xs) stv<W>(px3, xo, q3);
     if constexpr (YZ) c = dif<W>(xz, zx);
-    else c = mad<W>(xz, ihz, neg<W>(zx));
+    else c = mulsub<W>(false, xz, ihz, zx);
     Vec<W> e1 = mad<W>(c, c1, eo1);
     // Ez at (i, j, k+1/2)
     Vec<W> yx = mul<W>(dif<W>(hyc, hyx), r.ihx), xy = dif<W>(hxc, hxj);
@@ -423,7 +439,7 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
         xy = mul<W>(xy, r.ihy);
         if (ys) { cpml<W>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
         c = dif<W>(yx, xy);
-    } else c = mad<W>(xy, -r.ihy, yx);
+    } else c = submul<W>(!last, yx, xy, r.ihy);
     Vec<W> e2 = mad<W>(c, c2, eo2);
 
     if (taps) {
@@ -477,8 +493,8 @@ __device__ __forceinline__ void e_tile(const StepParams<float> &p, const int jst
         const int k = k0 + kk;
         if (k >= k1) break;
         if (yblk || k < npml || k > p.nz - npml)
-            e_plane<W, true, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, o, xo, oj, oi, taps, hxm, hym);
-        else e_plane<W, false, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, o, xo, oj, oi, taps, hxm, hym);
+            e_plane<W, true, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, kk == KZ - 1, o, xo, oj, oi, taps, hxm, hym);
+        else e_plane<W, false, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, kk == KZ - 1, o, xo, oj, oi, taps, hxm, hym);
     }
 }
 
@@ -519,8 +535,9 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepPa
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        if (yblk || k < npml || k > p.nz - npml) e_plane<W, true, false>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, o, xo, oj, oi, taps, hxm, hym);
-        else e_plane<W, false, false>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, o, xo, oj, oi, taps, hxm, hym);
+        const bool last = TAIL ? (k & (KZ - 1)) == KZ - 1 : kk == KZ - 1;   // z blocks start at multiples of KZ without big_blocks
+        if (yblk || k < npml || k > p.nz - npml) e_plane<W, true, false>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
+        else e_plane<W, false, false>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
     }
 }
 

@@ -1,0 +1,55 @@
+"""Roundings of the FP32 step kernels.  Gradients multiply a rounding difference by up to 10^4 (the adjoint basis is
+ill-conditioned), so the kernels spell their roundings out: traces equal the stored ones of the same kernels compiled
+from plain expressions, and every instance with the same planes per thread gives the same bits."""
+import json
+import os
+
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2211_16665_gb300 import workloads as W  # noqa: E402
+
+GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "step_roundings.json")
+CONFIGS = {"order 2, %d planes" % kz: dict(order=2, kz=kz, mb=6) for kz in (1, 2, 4)}
+
+
+def trace_of(order, kz, mb):
+    """Traces of a 44^3 box with graded cells, every fourth step: [receiver][step], FP64 sums of FP32 field values."""
+    from paper_2211_16665_gb300.engine import Engine
+    wl = W.small_box(n_core=20, n_st=4, ratio=1.05, npml=8, n_freq=2, nt=160, n_rec=3)
+    eng = Engine.from_workload(wl, max_src=1, autotune=False, order=order)
+    eng.set_launch(kz_h=kz, mb_h=mb, lean_h=2, kz_e=kz, mb_e=mb, lean_e=2)
+    tr = eng.fwd_model(eng.model_tensor(wl.rho_true), wl.src, wl.rec, trace=True)[-1]
+    eng.check()
+    eng.close()
+    return tr[0, :, 3::4].cpu()
+
+
+@pytest.mark.parametrize("name", CONFIGS)
+def test_traces_are_what_they_were(name):
+    tr = trace_of(**CONFIGS[name])
+    with open(GOLDEN) as f:
+        want = torch.tensor(json.load(f)[name], dtype=torch.float64)
+    assert want.abs().max() > 0
+    # equal field bits leave the order and fusion of eight FP64 products: 16 roundings of 1.1e-16 of terms that are of
+    # the order of the trace's peak.  One FP32 rounding on the way is 6e-8 of a value, 1e-3 of the peak or more.
+    assert ((tr - want).abs().amax(-1) <= 1e-13 * want.abs().amax(-1)).all()
+
+
+# 96 x 88 x 90 cells: some of these launches end in one-plane blocks (1.2 to 8 waves), the others do not
+@pytest.mark.parametrize("kz", [1, 2, 4])
+def test_instances_give_the_same_bits(kz):
+    from paper_2211_16665_gb300.engine import Engine
+    wl = W.small_box(n_core=84, n_core_y=76, n_core_z=78, npml=6, n_freq=2, nt=64, n_rec=4)
+    out = []
+    for w, mb in ((1, 6), (1, 8), (2, 4), (2, 6), (2, 8)):
+        eng = Engine.from_workload(wl, max_src=1, autotune=False)
+        eng.set_launch(kz_h=kz, mb_h=mb, lean_h=w, kz_e=kz, mb_e=mb, lean_e=w)
+        d, E = eng.fwd_model(eng.model_tensor(wl.rho_true), wl.src, wl.rec, keep_volume=True)
+        eng.check()
+        eng.close()
+        out.append((d, E))
+    for d, E in out[1:]:
+        assert torch.equal(d, out[0][0]) and torch.equal(E, out[0][1])
