@@ -1406,7 +1406,7 @@ int autotune_impl(csem_ctx *c, int S, cudaStream_t st) {
                 const int bm[4][2] = {{4, 4}, {4, 6}, {8, 2}, {8, 3}};
                 for (const auto &b : bm)
                     for (int kz : {8, 16, 32, 64}) cands.push_back({0, b[0], b[1], kz, 0, 0});
-                if (c->d_cEm && c->d_psi) {        // the warp-specialised fused step
+                if (c->d_cEm && c->d_psi && c->nx % 4 == 0) {        // the warp-specialised fused step
                     const int wm[5][2] = {{4, 2}, {4, 3}, {6, 2}, {8, 1}, {8, 2}};
                     for (const auto &b : wm)
                         for (int kz : {8, 16, 32, 64}) cands.push_back({0, b[0], b[1], kz, 1, 0});
@@ -1954,7 +1954,7 @@ int csem_set_launch(csem_ctx *c, const int *cfg) {
     const int fz_kz = fz / 100, fz_by = (fz / 10) % 10, fz_mb = fz % 10;
     if (fz && !ws && (c->precision != 32 || c->order != 2 || !c->d_q || c->nx % 2 != 0 || !csem::fz_supported(fz_by, fz_mb, fz_kz)))
         return fail(CSEM_ERR_INVALID_ARG, "fused one-pass step: FP32, second order, nx even, rows/blocks (4,4), (4,6), (8,2) or (8,3), 2-99 planes");
-    if (ws && (c->precision != 32 || c->order != 2 || !c->d_q || !c->d_cEm || !c->d_psi || c->nx % 2 != 0 ||
+    if (ws && (c->precision != 32 || c->order != 2 || !c->d_q || !c->d_cEm || !c->d_psi || c->nx % 4 != 0 ||
                !csem::ws_supported(fz_by, fz_mb, fz_kz)))
         return fail(CSEM_ERR_INVALID_ARG, "warp-specialised fused step: FP32, second order, nx a multiple of 4, rows/blocks (4,2), (4,3), (6,2), (8,1) or (8,2), 2-99 planes");
     const int vh = cfg[7], ve = cfg[8], th = cfg[9], te = cfg[10], lh = cfg[11], le = cfg[12];
