@@ -321,7 +321,10 @@ int csem_set_early_stop_volumes(csem_ctx *ctx, double tol, double floor_frac);
  * csem_set_launch), then the step's form: 0 split, 4/8/16 the fused z
  * blocking, 10000 + code the one-pass kernel, 30000 + code the
  * warp-specialised fused kernel, 50000 + code the wave-ordered step.  Overwrites the
- * context's field state and blocks until the timing is done.
+ * context's field state and blocks until the timing is done.  In an FP32
+ * second-order context whose nx is no multiple of 4 the first call allocates
+ * the lean kernels' memory (12 volume arrays per source and three more) where
+ * it fits in a quarter of the free memory.
  * Errors: INVALID_ARG, CUDA. */
 int csem_autotune(csem_ctx *ctx, int n_src, int *kz_out, void *stream);
 
@@ -346,8 +349,8 @@ int csem_autotune(csem_ctx *ctx, int n_src, int *kz_out, void *stream);
  * E four-cells-per-thread (0/1), H bulk-copy-staged rows per block (0, or
  * 1/2/4 for FP32 when the staged planes fit shared memory; z planes 2-16),
  * E bulk-copy-staged rows per block, H lean kernel (0 off, or 1 or 2 cells
- * per thread: FP32 with nx a multiple of 4 and room for the CPML memory in 12
- * volume arrays per source; 1, 2 or 4 planes; blocks of 128 threads, 6 or 8
+ * per thread: FP32 with room for the CPML memory in 12 volume arrays per source,
+ * and nx a multiple of 4 or a context that csem_autotune has tuned; 1, 2 or 4 planes; blocks of 128 threads, 6 or 8
  * resident per SM, or 4, 6 or 8 with 2 cells), E lean kernel (0, 1 or 2)}
  * -- 13 ints.  The
  * lean kernel takes precedence over the staged and four-cell ones.

@@ -293,6 +293,29 @@ int upload_lean_tables(csem_ctx *c) {
     return CSEM_OK;
 }
 
+// Tap increments, tap planes and padded tables of the kernels that take a chunk's increments.
+int lean_small(csem_ctx *c) {
+    const int S = c->max_src, NR = std::max(c->max_rec, 1);
+    if (!c->d_inc) TRY(dalloc(c, &c->d_inc, (size_t)kChunk * S * std::max(8, NR * 8) * sizeof(float)));
+    if (!c->d_tapk) TRY(dalloc(c, &c->d_tapk, (size_t)std::max(S, NR) * 8 * sizeof(int)));
+    return c->d_tabL ? CSEM_OK : upload_lean_tables(c);
+}
+// The volumes of the lean split kernels (FP32, second order): the CPML memory in 12 volume arrays per source and the
+// masked dt/eps.  They are taken where they fit in a quarter of the free memory (the kernels' byte offsets are 32 bits).
+bool lean_fits(const csem_ctx *c) {
+    size_t free_b = 0, total_b = 0;
+    cudaMemGetInfo(&free_b, &total_b);
+    const double need = ((double)c->max_src * 12 + 3) * c->vol * sizeof(float);
+    return c->vol < (1LL << 30) && need < 0.25 * (double)free_b;
+}
+int lean_memory(csem_ctx *c) {
+    if (!c->d_cEm) {
+        TRY(dalloc(c, &c->d_cEm, 3 * (size_t)c->vol * sizeof(float)));
+        CK(cudaMemset(c->d_cEm, 0, 3 * (size_t)c->vol * sizeof(float)));
+    }
+    return dalloc(c, &c->d_psiL, (size_t)c->max_src * 12 * c->vol * sizeof(float));
+}
+
 template <typename R>
 int upload_tables(csem_ctx *c) {
     std::vector<R> tab;
@@ -1319,6 +1342,14 @@ int time_impl(csem_ctx *c, int S, void *vol, int launches, double *ms, cudaStrea
 // Times the H and E kernels for every z-blocking candidate on S sources and keeps the fastest.
 template <typename R>
 int autotune_impl(csem_ctx *c, int S, cudaStream_t st) {
+    // rows that are no multiple of four: only the autotuner brings the lean kernels there, so it takes their memory
+    // (without it they are not among the candidates)
+    if (sizeof(R) == 4 && c->order == 2 && !c->d_psiL && c->nx % 4 != 0 && lean_fits(c)) {
+        int rc = lean_small(c);
+        if (rc == CSEM_OK) rc = lean_memory(c);
+        if (rc != CSEM_OK && rc != CSEM_ERR_OOM) return rc;
+        CK(cudaDeviceSynchronize());     // the tables and zeros are in place before the stream reads them
+    }
     TRY(reset_state<R>(c, S, st));
     c->ring_dirty = true;                // every kernel family steps in the ring
     csem::StepParams<R> p = step_params<R>(c, false, nullptr);
@@ -1697,16 +1728,16 @@ int csem_create(csem_ctx **out, const csem_grid *g, const csem_opts *o) {
                 rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
         }
     }
-    // FP32: tap increments, padded tables and the masked dt/eps of the lean kernels (fourth order: nx even);
-    // second order also the CPML memory of the lean split kernels in 12 volume arrays per source, kept when it
-    // fits, and, nx even, the fused one-pass step's per-cell material and widths
-    if (rc == CSEM_OK && c->precision == 32 && (c->order == 2 || (c->nx % 2 == 0 && c->vol < (1LL << 30)))) {
-        step(dalloc(c, &c->d_inc, (size_t)kChunk * S * std::max(8, NR * 8) * sizeof(float)));
-        step(dalloc(c, &c->d_tapk, (size_t)std::max(S, NR) * 8 * sizeof(int)));
-        step(upload_lean_tables(c));
-        step(dalloc(c, &c->d_cEm, 3 * (size_t)c->vol * sizeof(float)));
-        if (rc == CSEM_OK && cudaMemset(c->d_cEm, 0, 3 * (size_t)c->vol * sizeof(float)) != cudaSuccess)
-            rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
+    // FP32, nx even: tap increments and padded tables (and for the fourth order the masked dt/eps of its lean
+    // kernels); second order also the fused one-pass step's per-cell material and widths, and with nx a multiple
+    // of 4 the memory of the lean split kernels (on other rows csem_autotune takes it)
+    if (rc == CSEM_OK && c->precision == 32 && c->nx % 2 == 0 && (c->order == 2 || c->vol < (1LL << 30))) {
+        step(lean_small(c));
+        if (c->order == 4) {
+            step(dalloc(c, &c->d_cEm, 3 * (size_t)c->vol * sizeof(float)));
+            if (rc == CSEM_OK && cudaMemset(c->d_cEm, 0, 3 * (size_t)c->vol * sizeof(float)) != cudaSuccess)
+                rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
+        }
     }
     if (rc == CSEM_OK && c->order == 2 && c->precision == 32 && c->nx % 2 == 0) {
         if (rc == CSEM_OK) step(upload_geo_tables(c));
@@ -1717,16 +1748,11 @@ int csem_create(csem_ctx **out, const csem_grid *g, const csem_opts *o) {
         if (rc == CSEM_OK && cudaMemset(c->d_q, 0x3f, qb) != cudaSuccess)
             rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
     }
-    if (rc == CSEM_OK && c->order == 2 && c->precision == 32) {
-        size_t free_b = 0, total_b = 0;
-        cudaMemGetInfo(&free_b, &total_b);
-        const double need = (double)S * 12 * c->vol * sizeof(float);
-        if (need < 0.25 * (double)free_b && c->vol < (1LL << 30)) {   // the kernels' byte offsets are 32 bits
-            step(dalloc(c, &c->d_psiL, (size_t)S * 12 * c->vol * sizeof(float)));
-            if (c->nx % 4 == 0) step(dalloc(c, &c->d_wave, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)));
-            if (rc == CSEM_OK && c->d_wave && cudaMemset(c->d_wave, 0, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)) != cudaSuccess)
-                rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
-        }
+    if (c->order == 2 && c->precision == 32 && c->nx % 4 == 0) {
+        if (rc == CSEM_OK && lean_fits(c)) step(lean_memory(c));
+        if (c->d_psiL) step(dalloc(c, &c->d_wave, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)));
+        if (rc == CSEM_OK && c->d_wave && cudaMemset(c->d_wave, 0, (2 + csem::kMaxWaveChunks) * sizeof(unsigned)) != cudaSuccess)
+            rc = fail(CSEM_ERR_CUDA, "context initialisation failed");
     }
     if (rc != CSEM_OK) { free_ctx(c); return rc; }
     std::vector<double> hcat;
@@ -1978,8 +2004,8 @@ int csem_set_launch(csem_ctx *c, const int *cfg) {
             return l == 0 || ((l == 1 || l == 2) && (kz == 1 || kz == 2 || kz == 4) &&
                               (mb == 6 || mb == 8 || (mb == 4 && l == 2)));
         };
-        if (!c->d_psiL || c->nx % 4 != 0 || !ok(lh, kzh, mbh) || !ok(le, kze, mbe))
-            return fail(CSEM_ERR_INVALID_ARG, "lean kernels: FP32, nx a multiple of 4, 1 or 2 cells, 1/2/4 planes, 6 or 8 (2 cells: 4, 6 or 8) blocks/SM");
+        if (!c->d_psiL || !ok(lh, kzh, mbh) || !ok(le, kze, mbe))
+            return fail(CSEM_ERR_INVALID_ARG, "lean kernels: FP32, nx a multiple of 4 (or a tuned context), 1 or 2 cells, 1/2/4 planes, 6 or 8 (2 cells: 4, 6 or 8) blocks/SM");
     }
     if (th || te) {
         const int maxty = c->precision == 32 ? csem::tma_max_rows(c->pitch) : 0;
