@@ -143,18 +143,19 @@ template <int W> __device__ __forceinline__ Vec<W> neg(const Vec<W> &a) {
     for (int e = 0; e < W; ++e) r.v[e] = -a.v[e];
     return r;
 }
-// CPML recursion psi <- b psi + a d, then d += psi (shared or per-cell b, a); b psi is fused to the rounded a d.
-__device__ __forceinline__ void cpml1(float &ps, float &d, float b, float a) {
-    ps = fmaf(b, ps, __fmul_rn(a, d));
+// CPML recursion psi <- b psi + a d, then d += psi (shared or per-cell b, a).  BF: b psi is fused to the rounded a d,
+// else a d to the rounded b psi.
+template <bool BF> __device__ __forceinline__ void cpml1(float &ps, float &d, float b, float a) {
+    ps = BF ? fmaf(b, ps, __fmul_rn(a, d)) : fmaf(a, d, __fmul_rn(b, ps));
     d = __fadd_rn(d, ps);
 }
-template <int W> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, float b, float a) {
+template <int W, bool BF> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, float b, float a) {
 #pragma unroll
-    for (int e = 0; e < W; ++e) cpml1(ps.v[e], d.v[e], b, a);
+    for (int e = 0; e < W; ++e) cpml1<BF>(ps.v[e], d.v[e], b, a);
 }
-template <int W> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, const Vec<W> &b, const Vec<W> &a) {
+template <int W, bool BF> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, const Vec<W> &b, const Vec<W> &a) {
 #pragma unroll
-    for (int e = 0; e < W; ++e) cpml1(ps.v[e], d.v[e], b.v[e], a.v[e]);
+    for (int e = 0; e < W; ++e) cpml1<BF>(ps.v[e], d.v[e], b.v[e], a.v[e]);
 }
 // u s - v and v - u s, the product rounded first or (fuse) fused to v
 template <int W> __device__ __forceinline__ Vec<W> mulsub(bool fuse, const Vec<W> &u, float s, const Vec<W> &v) {
@@ -226,10 +227,12 @@ __device__ __forceinline__ float3 lean_taps(const int *__restrict__ tk, const fl
 }  // namespace
 
 // One plane k of the H update for the thread's W cells; YZ: the y/z recursion
-// may apply (a block on a y or z slab); FAR: see kFarBytes.  Off the slabs the products
-// of a difference are fused, but for those of Hy and Hz in the last plane of a z block of KZ planes (last).  o: byte offset of the cells in a component,
-// xo: of their x-slab entries.  exc, eyc: Ex, Ey of plane k (in), of plane k+1 (out).
-template <int W, bool YZ, bool FAR>
+// may apply (a block on a y or z slab); FAR: see kFarBytes.  F4: the row length is a multiple of four; there the
+// products of a difference off the slabs are fused, but for those of Hy and Hz in the last plane of a z block of KZ
+// planes (last), and b psi is fused in the recursions.  Other rows ran the four-cell H and the scalar E kernel before
+// the lean ones took them, and keep the roundings of those: no fused product off the slabs, in H b psi fused along x
+// and a d along y and z, in E a d.  o: byte offset of the cells in a component, xo: of their x-slab entries.  exc, eyc: Ex, Ey of plane k (in), of plane k+1 (out).
+template <int W, bool YZ, bool FAR, bool F4>
 __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float *__restrict__ E, float *__restrict__ H,
                                         float *__restrict__ ps, const LeanRow<W> &r, int k, bool last, unsigned o, unsigned xo,
                                         Vec<W> &exc, Vec<W> &eyc) {
@@ -263,31 +266,31 @@ __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float 
     Vec<W> zy = dif<W>(ezj, ezc), yz = dif<W>(eyk, eyc), c;
     if constexpr (YZ) {
         zy = mul<W>(zy, r.ihy); yz = mul<W>(yz, ihz);
-        if (ys) { cpml<W>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
-        if (zs) { cpml<W>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
+        if (ys) { cpml<W, F4>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
+        if (zs) { cpml<W, F4>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
         c = dif<W>(zy, yz);
-    } else c = mulsub<W>(true, zy, r.ihy, mul<W>(yz, ihz));
+    } else c = mulsub<W>(F4, zy, r.ihy, mul<W>(yz, ihz));
     hx = mad<W>(c, -p.cH, hx);
     // Hy at (i+1/2, j, k+1/2)
     Vec<W> xz = dif<W>(exk, exc), zx = mul<W>(dif<W>(ezx, ezc), r.ihx);
     if constexpr (YZ) {
         xz = mul<W>(xz, ihz);
-        if (zs) { cpml<W>(q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
+        if (zs) { cpml<W, F4>(q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
     }
-    cpml<W>(q3, zx, r.bx, r.ax);
+    cpml<W, true>(q3, zx, r.bx, r.ax);
     if (r.xs) stv<W>(px3, xo, q3);
     if constexpr (YZ) c = dif<W>(xz, zx);
-    else c = mulsub<W>(!last, xz, ihz, zx);
+    else c = mulsub<W>(F4 && !last, xz, ihz, zx);
     hy = mad<W>(c, -p.cH, hy);
     // Hz at (i+1/2, j+1/2, k)
     Vec<W> yx = mul<W>(dif<W>(eyx, eyc), r.ihx), xy = dif<W>(exj, exc);
-    cpml<W>(q4, yx, r.bx, r.ax);
+    cpml<W, true>(q4, yx, r.bx, r.ax);
     if (r.xs) stv<W>(px4, xo, q4);
     if constexpr (YZ) {
         xy = mul<W>(xy, r.ihy);
-        if (ys) { cpml<W>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
+        if (ys) { cpml<W, F4>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
         c = dif<W>(yx, xy);
-    } else c = submul<W>(!last, yx, xy, r.ihy);
+    } else c = submul<W>(F4 && !last, yx, xy, r.ihy);
     hz = mad<W>(c, -p.cH, hz);
 
     if constexpr (FAR) { stl<W>(H, o, hx); stl<W>(Hy, o, hy); stl<W>(Hz, o, hz); }
@@ -324,12 +327,12 @@ __device__ __forceinline__ void h_tile(const StepParams<float> &p, const int jst
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, false>(p, E, H, ps, r, k, kk == KZ - 1, o, xo, exc, eyc);
-        else h_plane<W, false, false>(p, E, H, ps, r, k, kk == KZ - 1, o, xo, exc, eyc);
+        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, false, true>(p, E, H, ps, r, k, kk == KZ - 1, o, xo, exc, eyc);
+        else h_plane<W, false, false, true>(p, E, H, ps, r, k, kk == KZ - 1, o, xo, exc, eyc);
     }
 }
 
-template <int W, int KZ, int MINB, bool FAR, bool TAIL>
+template <int W, int KZ, int MINB, bool FAR, bool TAIL, bool F4>
 __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepParams<float> p, const int jstep, const unsigned S,
                                                                        const unsigned mS, const int nbig) {
     const int i = (blockIdx.x * kLeanX + threadIdx.x) * W;
@@ -358,9 +361,9 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepPa
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        const bool last = TAIL ? (k & (KZ - 1)) == KZ - 1 : kk == KZ - 1;   // z blocks start at multiples of KZ without big_blocks
-        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, FAR>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
-        else h_plane<W, false, FAR>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
+        const bool last = TAIL ? (k & (KZ - 1)) == KZ - 1 : kk == KZ - 1;   // without big_blocks z blocks start at multiples of KZ
+        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, FAR, F4>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
+        else h_plane<W, false, FAR, F4>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
     }
 }
 
@@ -380,8 +383,9 @@ template <bool CG> __device__ __forceinline__ float ldh1(const float *b, unsigne
 }
 
 // One plane k of the E update; o, xo as in h_plane; oj, oi: from o to the lower neighbours along y and x (0 on
-// the outer faces).  hxm, hym: Hx, Hy of plane k-1 (in), of plane k (out).
-template <int W, bool YZ, bool CG>
+// the outer faces).  F4: off the slabs Ey's products are never fused, Ez's not in the last plane.  hxm, hym: Hx, Hy of
+// plane k-1 (in), of plane k (out).
+template <int W, bool YZ, bool CG, bool F4>
 __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float *__restrict__ Eo, float *__restrict__ En,
                                         const float *__restrict__ H, float *__restrict__ ps, const LeanRow<W> &r, int s,
                                         int S, int jstep, int k, bool last, unsigned o, unsigned xo, unsigned oj,
@@ -415,31 +419,31 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
     Vec<W> zy = dif<W>(hzc, hzj), yz = dif<W>(hyc, hym), c;
     if constexpr (YZ) {
         zy = mul<W>(zy, r.ihy); yz = mul<W>(yz, ihz);
-        if (ys) { cpml<W>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
-        if (zs) { cpml<W>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
+        if (ys) { cpml<W, F4>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
+        if (zs) { cpml<W, F4>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
         c = dif<W>(zy, yz);
-    } else c = mulsub<W>(true, zy, r.ihy, mul<W>(yz, ihz));
+    } else c = mulsub<W>(F4, zy, r.ihy, mul<W>(yz, ihz));
     Vec<W> e0 = mad<W>(c, c0, eo0);
     // Ey at (i, j+1/2, k)
     Vec<W> xz = dif<W>(hxc, hxm), zx = mul<W>(dif<W>(hzc, hzx), r.ihx);
     if constexpr (YZ) {
         xz = mul<W>(xz, ihz);
-        if (zs) { cpml<W>(q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
+        if (zs) { cpml<W, F4>(q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
     }
-    cpml<W>(q3, zx, r.bx, r.ax);
+    cpml<W, F4>(q3, zx, r.bx, r.ax);
     if (r.xs) stv<W>(px3, xo, q3);
     if constexpr (YZ) c = dif<W>(xz, zx);
     else c = mulsub<W>(false, xz, ihz, zx);
     Vec<W> e1 = mad<W>(c, c1, eo1);
     // Ez at (i, j, k+1/2)
     Vec<W> yx = mul<W>(dif<W>(hyc, hyx), r.ihx), xy = dif<W>(hxc, hxj);
-    cpml<W>(q4, yx, r.bx, r.ax);
+    cpml<W, F4>(q4, yx, r.bx, r.ax);
     if (r.xs) stv<W>(px4, xo, q4);
     if constexpr (YZ) {
         xy = mul<W>(xy, r.ihy);
-        if (ys) { cpml<W>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
+        if (ys) { cpml<W, F4>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
         c = dif<W>(yx, xy);
-    } else c = submul<W>(!last, yx, xy, r.ihy);
+    } else c = submul<W>(F4 && !last, yx, xy, r.ihy);
     Vec<W> e2 = mad<W>(c, c2, eo2);
 
     if (taps) {
@@ -493,12 +497,12 @@ __device__ __forceinline__ void e_tile(const StepParams<float> &p, const int jst
         const int k = k0 + kk;
         if (k >= k1) break;
         if (yblk || k < npml || k > p.nz - npml)
-            e_plane<W, true, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, kk == KZ - 1, o, xo, oj, oi, taps, hxm, hym);
-        else e_plane<W, false, CG>(p, Eo, En, H, ps, r, s, S, jstep, k, kk == KZ - 1, o, xo, oj, oi, taps, hxm, hym);
+            e_plane<W, true, CG, true>(p, Eo, En, H, ps, r, s, S, jstep, k, kk == KZ - 1, o, xo, oj, oi, taps, hxm, hym);
+        else e_plane<W, false, CG, true>(p, Eo, En, H, ps, r, s, S, jstep, k, kk == KZ - 1, o, xo, oj, oi, taps, hxm, hym);
     }
 }
 
-template <int W, int KZ, int MINB, bool FAR, bool TAIL>
+template <int W, int KZ, int MINB, bool FAR, bool TAIL, bool F4>
 __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepParams<float> p, const int jstep, const unsigned S,
                                                                        const unsigned mS, const int nbig) {
     const int i = (blockIdx.x * kLeanX + threadIdx.x) * W;
@@ -535,9 +539,9 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepPa
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        const bool last = TAIL ? (k & (KZ - 1)) == KZ - 1 : kk == KZ - 1;   // z blocks start at multiples of KZ without big_blocks
-        if (yblk || k < npml || k > p.nz - npml) e_plane<W, true, false>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
-        else e_plane<W, false, false>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
+        const bool last = TAIL ? (k & (KZ - 1)) == KZ - 1 : kk == KZ - 1;   // without big_blocks z blocks start at multiples of KZ
+        if (yblk || k < npml || k > p.nz - npml) e_plane<W, true, false, F4>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
+        else e_plane<W, false, false, F4>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
     }
 }
 
@@ -682,31 +686,36 @@ __global__ void k_mask_coef(const StepParams<float> p, const float *__restrict__
 }
 
 namespace {
-template <int W, int KZ, int MB, bool TAIL>
+template <int W, int KZ, int MB, bool TAIL, bool F4>
 void lean_launch(const StepParams<float> &p, dim3 grid, int nbig, int S, int jstep, cudaStream_t st, bool h) {
     const dim3 block(kLeanX, kLeanRows);
     const unsigned mS = div_magic((unsigned)S);
     const bool far = far_fields(p.vol, S);
-    if (h && far) launch_pdl(k_h_lean<W, KZ, MB, true, TAIL>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
-    else if (h) launch_pdl(k_h_lean<W, KZ, MB, false, TAIL>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
-    else if (far) launch_pdl(k_e_lean<W, KZ, MB, true, TAIL>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
-    else launch_pdl(k_e_lean<W, KZ, MB, false, TAIL>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+    if (h && far) launch_pdl(k_h_lean<W, KZ, MB, true, TAIL, F4>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+    else if (h) launch_pdl(k_h_lean<W, KZ, MB, false, TAIL, F4>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+    else if (far) launch_pdl(k_e_lean<W, KZ, MB, true, TAIL, F4>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+    else launch_pdl(k_e_lean<W, KZ, MB, false, TAIL, F4>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
 }
-template <int W, int KZ, int MB>
+template <int W, int KZ, int MB, bool F4>
 void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h) {
     const int nv = (p.nx + W - 1) / W, nzb = (p.nz + KZ - 1) / KZ;
     const int gx = (nv + kLeanX - 1) / kLeanX, gy = (p.ny + kLeanRows - 1) / kLeanRows;
     const int nbig = big_blocks(nzb, KZ, gx * gy * S, MB);
     if constexpr (KZ > 1)
-        if (nbig < nzb) return lean_launch<W, KZ, MB, true>(p, dim3(gx, gy, (nbig + p.nz - nbig * KZ) * S), nbig, S, jstep, st, h);
-    lean_launch<W, KZ, MB, false>(p, dim3(gx, gy, nzb * S), nzb, S, jstep, st, h);
+        if (nbig < nzb) return lean_launch<W, KZ, MB, true, F4>(p, dim3(gx, gy, (nbig + p.nz - nbig * KZ) * S), nbig, S, jstep, st, h);
+    lean_launch<W, KZ, MB, false, F4>(p, dim3(gx, gy, nzb * S), nzb, S, jstep, st, h);
+}
+template <int W, int KZ, int MB>
+void lean_rows(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h) {
+    if (p.nx % 4 == 0) lean_go<W, KZ, MB, true>(p, S, jstep, st, h);
+    else lean_go<W, KZ, MB, false>(p, S, jstep, st, h);
 }
 template <int W, int MB>
 bool lean_kz(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int kz) {
     switch (kz) {
-        case 1: lean_go<W, 1, MB>(p, S, jstep, st, h); return true;
-        case 2: lean_go<W, 2, MB>(p, S, jstep, st, h); return true;
-        case 4: lean_go<W, 4, MB>(p, S, jstep, st, h); return true;
+        case 1: lean_rows<W, 1, MB>(p, S, jstep, st, h); return true;
+        case 2: lean_rows<W, 2, MB>(p, S, jstep, st, h); return true;
+        case 4: lean_rows<W, 4, MB>(p, S, jstep, st, h); return true;
         default: return false;
     }
 }
