@@ -17,13 +17,26 @@ constexpr int kHoX = 32, kHoY = 8, kHoZ = 4;
 
 template <typename R> __device__ __forceinline__ R ld(const R *p) { return __ldg(p); }
 
+// The roundings are spelled out: left to itself the compiler fuses one product or the other of a sum of two, and
+// another one with every change of a kernel; gradients multiply such a difference by up to 10^4.  The choices are
+// those of the kernels as first compiled from plain expressions, so results are what they were.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+// a b + c d: a b fused to the rounded c d
+template <typename R> __device__ __forceinline__ R dot2(R a, R b, R c, R d) { return fma_rn(a, b, mul_rn(c, d)); }
+
+
 // d/da at the half node pos (of n) of a node-located field F, F[at] at node pos
 template <typename R>
 __device__ __forceinline__ R d_half(const R *__restrict__ F, long long at, long long s, int pos, int n,
                                     const R *__restrict__ w) {
     const R *wr = w + 4 * pos;
-    R d = ld(wr + 1) * ld(F + at) + ld(wr + 2) * ld(F + at + s);
-    if (pos >= 1 && pos <= n - 2) d = ld(wr) * ld(F + at - s) + d + ld(wr + 3) * ld(F + at + 2 * s);
+    R d = dot2(ld(wr + 1), ld(F + at), ld(wr + 2), ld(F + at + s));
+    if (pos >= 1 && pos <= n - 2) d = fma_rn(ld(wr + 3), ld(F + at + 2 * s), fma_rn(ld(wr), ld(F + at - s), d));
     return d;
 }
 
@@ -32,8 +45,8 @@ template <typename R>
 __device__ __forceinline__ R d_node(const R *F, long long at, long long s, int pos, int n,
                                     const R *__restrict__ w) {
     const R *wr = w + 4 * pos;
-    R d = ld(wr + 1) * F[at - s] + ld(wr + 2) * F[at];
-    if (pos >= 2 && pos <= n - 2) d = ld(wr) * F[at - 2 * s] + d + ld(wr + 3) * F[at + s];
+    R d = dot2(ld(wr + 1), F[at - s], ld(wr + 2), F[at]);
+    if (pos >= 2 && pos <= n - 2) d = fma_rn(ld(wr + 3), F[at + s], fma_rn(ld(wr), F[at - 2 * s], d));
     return d;
 }
 
@@ -41,9 +54,9 @@ __device__ __forceinline__ R d_node(const R *F, long long at, long long s, int p
 template <typename R>
 __device__ __forceinline__ R pml(R d, bool in, R b, R a, R q, R *ps) {
     if (!in) return d;
-    const R v = b * q + a * d;
+    const R v = dot2(a, d, b, q);
     *ps = v;
-    return d + v;
+    return add_rn(d, v);
 }
 
 template <typename R>
@@ -79,17 +92,17 @@ __global__ void __launch_bounds__(kHoX *kHoY) k_h_ho(const StepParams<R> p, cons
         if (j < ny && k < nz) {            // Hx at (i, j+1/2, k+1/2)
             const R a = pml(d_half(Ez, idx, pitch, j, ny, w.wyh), yin, by, ay_, q0, P + idx);
             const R b = pml(d_half(Ey, idx, plane, k, nz, w.wzh), zin, bz, az_, q1, P + vol + idx);
-            Hx[idx] -= cH * (a - b);
+            Hx[idx] = fma_rn(-cH, add_rn(a, -b), Hx[idx]);
         }
         if (i < nx && k < nz) {            // Hy at (i+1/2, j, k+1/2)
             const R a = pml(d_half(Ex, idx, plane, k, nz, w.wzh), zin, bz, az_, q2, P + 2 * vol + idx);
             const R b = pml(d_half(Ez, idx, 1LL, i, nx, w.wxh), xin, bx, ax_, q3, P + 3 * vol + idx);
-            Hy[idx] -= cH * (a - b);
+            Hy[idx] = fma_rn(-cH, add_rn(a, -b), Hy[idx]);
         }
         if (i < nx && j < ny) {            // Hz at (i+1/2, j+1/2, k)
             const R a = pml(d_half(Ey, idx, 1LL, i, nx, w.wxh), xin, bx, ax_, q4, P + 4 * vol + idx);
             const R b = pml(d_half(Ex, idx, pitch, j, ny, w.wyh), yin, by, ay_, q5, P + 5 * vol + idx);
-            Hz[idx] -= cH * (a - b);
+            Hz[idx] = fma_rn(-cH, add_rn(a, -b), Hz[idx]);
         }
     }
 }
@@ -127,17 +140,17 @@ __global__ void __launch_bounds__(kHoX *kHoY) k_e_ho(const StepParams<R> p, cons
         if (i < nx && jy && kz) {          // Ex at (i+1/2, j, k)
             const R a = pml(d_node(Hz, idx, pitch, j, ny, w.wyn), yin, by, ay_, q0, P + 6 * vol + idx);
             const R b = pml(d_node(Hy, idx, plane, k, nz, w.wzn), zin, bz, az_, q1, P + 7 * vol + idx);
-            En[idx] = ld(Eo + idx) + ld(p.cE + idx) * (a - b);
+            En[idx] = fma_rn(ld(p.cE + idx), add_rn(a, -b), ld(Eo + idx));
         }
         if (j < ny && ix && kz) {          // Ey at (i, j+1/2, k)
             const R a = pml(d_node(Hx, idx, plane, k, nz, w.wzn), zin, bz, az_, q2, P + 8 * vol + idx);
             const R b = pml(d_node(Hz, idx, 1LL, i, nx, w.wxn), xin, bx, ax_, q3, P + 9 * vol + idx);
-            En[vol + idx] = ld(Eo + vol + idx) + ld(p.cE + vol + idx) * (a - b);
+            En[vol + idx] = fma_rn(ld(p.cE + vol + idx), add_rn(a, -b), ld(Eo + vol + idx));
         }
         if (k < nz && ix && jy) {          // Ez at (i, j, k+1/2)
             const R a = pml(d_node(Hy, idx, 1LL, i, nx, w.wxn), xin, bx, ax_, q4, P + 10 * vol + idx);
             const R b = pml(d_node(Hx, idx, pitch, j, ny, w.wyn), yin, by, ay_, q5, P + 11 * vol + idx);
-            En[2 * vol + idx] = ld(Eo + 2 * vol + idx) + ld(p.cE + 2 * vol + idx) * (a - b);
+            En[2 * vol + idx] = fma_rn(ld(p.cE + 2 * vol + idx), add_rn(a, -b), ld(Eo + 2 * vol + idx));
         }
     }
     // source term E^{n+1} -= dt/eps J'^{n+1/2} for the taps of this column and planes
@@ -191,14 +204,24 @@ __device__ __forceinline__ float f1g(const float *b, unsigned o) { return __ldg(
 __device__ __forceinline__ float f1w(const float *b, unsigned o) { return *at(b, o); }
 __device__ __forceinline__ void f2s(float *b, unsigned o, float2 v) { f2s(const_cast<float *>(at(b, o)), v); }
 __device__ __forceinline__ float4 f4g(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
-// w . (a, b, c, d) for both cells of the pair
-__device__ __forceinline__ float2 dot4(const float4 &w, float2 a, float2 b, float2 c, float2 d) {
-    return make_float2(w.x * a.x + w.y * b.x + w.z * c.x + w.w * d.x, w.x * a.y + w.y * b.y + w.z * c.y + w.w * d.y);
+// w . (a, b, c, d); SEC: the second product is fused to the rounded first one, else the first to the rounded second
+template <bool SEC> __device__ __forceinline__ float dot4(const float4 &w, float a, float b, float c, float d) {
+    const float p = SEC ? dot2(w.y, b, w.x, a) : dot2(w.x, a, w.y, b);
+    return fma_rn(w.w, d, fma_rn(w.z, c, p));
+}
+// the same for both cells of the pair
+template <bool SEC> __device__ __forceinline__ float2 dot4(const float4 &w, float2 a, float2 b, float2 c, float2 d) {
+    return make_float2(dot4<SEC>(w, a.x, b.x, c.x, d.x), dot4<SEC>(w, a.y, b.y, c.y, d.y));
 }
 // x derivative of the pair from five consecutive values f0 .. f4 (cell i uses f0..f3, cell i+1 f1..f4)
+template <bool SEC0, bool SEC1>
 __device__ __forceinline__ float2 dx5(const float4 &w0, const float4 &w1, float f0, float f1, float f2, float f3,
                                       float f4) {
-    return make_float2(w0.x * f0 + w0.y * f1 + w0.z * f2 + w0.w * f3, w1.x * f1 + w1.y * f2 + w1.z * f3 + w1.w * f4);
+    return make_float2(dot4<SEC0>(w0, f0, f1, f2, f3), dot4<SEC1>(w1, f1, f2, f3, f4));
+}
+// h + c (u - v) for both cells
+__device__ __forceinline__ float2 curl2(float2 h, float2 c, float2 u, float2 v) {
+    return make_float2(fma_rn(c.x, add_rn(u.x, -v.x), h.x), fma_rn(c.y, add_rn(u.y, -v.y), h.y));
 }
 // d with its CPML memory v.  The six entries of a plane are loaded together (H: with the plane's fields; E: after
 // its differences, which leaves the registers of the fields for them).  Loaded one by one, each after the store of
@@ -206,15 +229,15 @@ __device__ __forceinline__ float2 dx5(const float4 &w0, const float4 &w1, float 
 // times per plane: 512 steps of 128 x 128 x 96, 25.6 -> 18.2 ms.
 __device__ __forceinline__ void pml2(float2 &d, bool in, float b, float a, float2 v, float *ps, unsigned o) {
     if (!in) return;
-    v.x = b * v.x + a * d.x; v.y = b * v.y + a * d.y;
+    v.x = dot2(a, d.x, b, v.x); v.y = dot2(a, d.y, b, v.y);
     f2s(ps, o, v);
-    d.x += v.x; d.y += v.y;
+    d.x = add_rn(d.x, v.x); d.y = add_rn(d.y, v.y);
 }
 __device__ __forceinline__ void pml2x(float2 &d, bool in, float2 b, float2 a, float2 v, float *ps, unsigned o) {
     if (!in) return;
-    v.x = b.x * v.x + a.x * d.x; v.y = b.y * v.y + a.y * d.y;
+    v.x = dot2(a.x, d.x, b.x, v.x); v.y = dot2(a.y, d.y, b.y, v.y);
     f2s(ps, o, v);
-    d.x += v.x; d.y += v.y;
+    d.x = add_rn(d.x, v.x); d.y = add_rn(d.y, v.y);
 }
 __device__ __forceinline__ float3 ho_taps(const int *__restrict__ tk, const float *__restrict__ inc, int k, int2 cm) {
     float3 r = make_float3(0.f, 0.f, 0.f);
@@ -247,7 +270,7 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
     const float *__restrict__ Ez = Ex + 2 * vol;
     float *__restrict__ H = p.H + (long long)s * 3 * vol;
     float *__restrict__ P = p.psi + (long long)s * p.psi_stride;
-    const float cH = p.cH;
+    const float2 mc = make_float2(-p.cH, -p.cH);
     // neighbours, clamped on the lattice: column i-1; rows j-1, j+2 (column i+3 lies in the
     // lattice row or its padding, and only the last half node's zero weight meets it there)
     const unsigned im = (i > 0) ? -4 : 0;
@@ -283,9 +306,9 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
         if (ys) { q0 = f2w(P, o); q5 = f2w(P + 5 * vol, o); }
         if (zs) { q1 = f2w(P + vol, o); q2 = f2w(P + 2 * vol, o); }
         if (xs) { q3 = f2w(P + 3 * vol, o); q4 = f2w(P + 4 * vol, o); }
-        float2 dEz_dy = dot4(wy, ezm2, ez01, ezp1, ezp2), dEy_dz = dot4(wz, ya, yb, yc, yd);
-        float2 dEx_dz = dot4(wz, xa, xb, xc, xd), dEz_dx = dx5(wx0, wx1, ezm, ez01.x, ez01.y, ez23.x, ez23.y);
-        float2 dEy_dx = dx5(wx0, wx1, eym, yb.x, yb.y, ey23.x, ey23.y), dEx_dy = dot4(wy, exm, xb, exp1, exp2);
+        float2 dEz_dy = dot4<true>(wy, ezm2, ez01, ezp1, ezp2), dEy_dz = dot4<false>(wz, ya, yb, yc, yd);
+        float2 dEx_dz = dot4<false>(wz, xa, xb, xc, xd), dEz_dx = dx5<false, false>(wx0, wx1, ezm, ez01.x, ez01.y, ez23.x, ez23.y);
+        float2 dEy_dx = dx5<true, false>(wx0, wx1, eym, yb.x, yb.y, ey23.x, ey23.y), dEx_dy = dot4<true>(wy, exm, xb, exp1, exp2);
         if (ys || zs || xs) {
             const float bz = __ldg(p.lz.b_h + k), az = __ldg(p.lz.a_h + k);
             pml2(dEz_dy, ys, by, ay, q0, P, o);
@@ -295,9 +318,9 @@ __global__ void __launch_bounds__(128, MINB) k_h_ho4(const StepParams<float> p, 
             pml2x(dEy_dx, xs, bx, ax, q4, P + 4 * vol, o);
             pml2(dEx_dy, ys, by, ay, q5, P + 5 * vol, o);
         }
-        hx.x -= cH * (dEz_dy.x - dEy_dz.x); hx.y -= cH * (dEz_dy.y - dEy_dz.y);
-        hy.x -= cH * (dEx_dz.x - dEz_dx.x); hy.y -= cH * (dEx_dz.y - dEz_dx.y);
-        hz.x -= cH * (dEy_dx.x - dEx_dy.x); hz.y -= cH * (dEy_dx.y - dEx_dy.y);
+        hx = curl2(hx, mc, dEz_dy, dEy_dz);
+        hy = curl2(hy, mc, dEx_dz, dEz_dx);
+        hz = curl2(hz, mc, dEy_dx, dEx_dy);
         f2s(H, o, hx);
         f2s(H + vol, o, hy);
         f2s(H + 2 * vol, o, hz);
@@ -361,11 +384,11 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
         const float2 e0 = f2e(Eo, o), e1 = f2e(Eo + vol, o), e2 = f2e(Eo + 2 * vol, o);
         const float2 c0 = f2g(cE, o), c1 = f2g(cE + vol, o), c2 = f2g(cE + 2 * vol, o);
         const bool zs = slab_node(k, nz, npml) >= 0;
-        float2 dHz_dy = dot4(wy, hzm2, hzm1, hz01, hzp1), dHy_dz = dot4(wz, ya, yb, yc, yd);
-        float2 dHx_dz = dot4(wz, xa, xb, xc, xd);
-        float2 dHz_dx = dx5(wx0, wx1, hzm.x, hzm.y, hz01.x, hz01.y, hz2);
-        float2 dHy_dx = dx5(wx0, wx1, hym.x, hym.y, yc.x, yc.y, hy2);
-        float2 dHx_dy = dot4(wy, hxm2, hxm1, xc, hxp1);
+        float2 dHz_dy = dot4<false>(wy, hzm2, hzm1, hz01, hzp1), dHy_dz = dot4<false>(wz, ya, yb, yc, yd);
+        float2 dHx_dz = dot4<false>(wz, xa, xb, xc, xd);
+        float2 dHz_dx = dx5<false, false>(wx0, wx1, hzm.x, hzm.y, hz01.x, hz01.y, hz2);
+        float2 dHy_dx = dx5<false, true>(wx0, wx1, hym.x, hym.y, yc.x, yc.y, hy2);
+        float2 dHx_dy = dot4<false>(wy, hxm2, hxm1, xc, hxp1);
         if (ys || zs || xs) {
             float2 q0 = {}, q1 = {}, q2 = {}, q3 = {}, q4 = {}, q5 = {};
             if (ys) { q0 = f2w(P, o); q5 = f2w(P + 5 * vol, o); }
@@ -379,9 +402,9 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
             pml2x(dHy_dx, xs, bx, ax, q4, P + 4 * vol, o);
             pml2(dHx_dy, ys, by, ay, q5, P + 5 * vol, o);
         }
-        float2 ex = make_float2(e0.x + c0.x * (dHz_dy.x - dHy_dz.x), e0.y + c0.y * (dHz_dy.y - dHy_dz.y));
-        float2 ey = make_float2(e1.x + c1.x * (dHx_dz.x - dHz_dx.x), e1.y + c1.y * (dHx_dz.y - dHz_dx.y));
-        float2 ez = make_float2(e2.x + c2.x * (dHy_dx.x - dHx_dy.x), e2.y + c2.y * (dHy_dx.y - dHx_dy.y));
+        float2 ex = curl2(e0, c0, dHz_dy, dHy_dz);
+        float2 ey = curl2(e1, c1, dHx_dz, dHz_dx);
+        float2 ez = curl2(e2, c2, dHy_dx, dHx_dy);
         if (taps) {
             const int2 *cm = p.colmap + (long long)s * p.colmap_stride + j * pitch + i;
             const int *tk = p.tapk + (long long)s * p.itap_stride;

@@ -13,14 +13,17 @@ from paper_2211_16665_gb300 import workloads as W  # noqa: E402
 
 GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "step_roundings.json")
 CONFIGS = {"order 2, %d planes" % kz: dict(order=2, kz=kz, mb=6) for kz in (1, 2, 4)}
+CONFIGS["order 4"] = dict(order=4, kz=4, mb=6)
+CONFIGS["order 4, odd rows"] = dict(order=4, kz=0, mb=0)        # nx = 45: the scalar kernels
 
 
 def trace_of(order, kz, mb):
     """Traces of a 44^3 box with graded cells, every fourth step: [receiver][step], FP64 sums of FP32 field values."""
     from paper_2211_16665_gb300.engine import Engine
-    wl = W.small_box(n_core=20, n_st=4, ratio=1.05, npml=8, n_freq=2, nt=160, n_rec=3)
+    wl = W.small_box(n_core=20 if mb else 21, n_st=4, ratio=1.05, npml=8, n_freq=2, nt=160, n_rec=3)
     eng = Engine.from_workload(wl, max_src=1, autotune=False, order=order)
-    eng.set_launch(kz_h=kz, mb_h=mb, lean_h=2, kz_e=kz, mb_e=mb, lean_e=2)
+    if mb:
+        eng.set_launch(kz_h=kz, mb_h=mb, lean_h=2, kz_e=kz, mb_e=mb, lean_e=2)
     tr = eng.fwd_model(eng.model_tensor(wl.rho_true), wl.src, wl.rec, trace=True)[-1]
     eng.check()
     eng.close()
@@ -51,6 +54,24 @@ def test_instances_give_the_same_bits(kz):
         eng.check()
         eng.close()
         out.append((d, E))
+    for d, E in out[1:]:
+        assert torch.equal(d, out[0][0]) and torch.equal(E, out[0][1])
+
+
+# Fourth order: the same bits for every planes per thread and blocks per SM, with and without one-plane blocks
+@pytest.mark.parametrize("nx", [96, 82])
+def test_fourth_order_instances_give_the_same_bits(nx):
+    from paper_2211_16665_gb300.engine import Engine
+    wl = W.small_box(n_core=nx - 12, n_core_y=76, n_core_z=78, npml=6, n_freq=2, nt=64, n_rec=4)
+    out = []
+    for kz in (2, 4, 8):
+        for mb in (4, 6, 8):
+            eng = Engine.from_workload(wl, max_src=1, autotune=False, order=4)
+            eng.set_launch(kz_h=kz, mb_h=mb, lean_h=2, kz_e=kz, mb_e=mb, lean_e=2)
+            d, E = eng.fwd_model(eng.model_tensor(wl.rho_true), wl.src, wl.rec, keep_volume=True)
+            eng.check()
+            eng.close()
+            out.append((d, E))
     for d, E in out[1:]:
         assert torch.equal(d, out[0][0]) and torch.equal(E, out[0][1])
 
