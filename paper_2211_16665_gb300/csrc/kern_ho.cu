@@ -119,9 +119,9 @@ __global__ void __launch_bounds__(kHoX *kHoY) k_e_ho(const StepParams<R> p, cons
     const long long vol = p.vol, plane = p.plane, pitch = p.pitch;
     const R *__restrict__ Eo = p.ering + (long long)s * p.ering_stride + (long long)(n % p.nslot) * 3 * vol;
     R *__restrict__ En = p.ering + (long long)s * p.ering_stride + (long long)((n + 1) % p.nslot) * 3 * vol;
-    const R *__restrict__ Hx = p.H + (long long)s * 3 * vol;
-    const R *__restrict__ Hy = Hx + vol;
-    const R *__restrict__ Hz = Hx + 2 * vol;
+    const R *Hx = p.H + (long long)s * 3 * vol;        // plain loads: see pdl_wait
+    const R *Hy = Hx + vol;
+    const R *Hz = Hx + 2 * vol;
     R *__restrict__ P = p.psi + (long long)s * p.psi_stride;
     const int nx = p.nx, ny = p.ny, nz = p.nz, npml = p.npml;
     const bool xin = slab_node(i, nx, npml) >= 0, yin = slab_node(j, ny, npml) >= 0;
@@ -347,9 +347,9 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
     const float *__restrict__ ring = p.ering + (long long)s * p.ering_stride;
     const float *__restrict__ Eo = ring + (long long)sl * 3 * p.vol;
     float *__restrict__ En = const_cast<float *>(ring) + (long long)slot_after(p, sl) * 3 * p.vol;
-    const float *__restrict__ Hx = p.H + (long long)s * 3 * vol;
-    const float *__restrict__ Hy = Hx + vol;
-    const float *__restrict__ Hz = Hx + 2 * vol;
+    const float *Hx = p.H + (long long)s * 3 * vol;        // plain loads: see pdl_wait
+    const float *Hy = Hx + vol;
+    const float *Hz = Hx + 2 * vol;
     float *__restrict__ P = p.psi + (long long)s * p.psi_stride + 6LL * vol;
     const float *__restrict__ cE = p.cEm;
     // neighbours, clamped on the lattice: columns i-2; rows j-2, j-1

@@ -387,7 +387,7 @@ template <bool CG> __device__ __forceinline__ float ldh1(const float *b, unsigne
 // plane k-1 (in), of plane k (out).
 template <int W, bool YZ, bool CG, bool F4>
 __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float *__restrict__ Eo, float *__restrict__ En,
-                                        const float *__restrict__ H, float *__restrict__ ps, const LeanRow<W> &r, int s,
+                                        const float *H, float *__restrict__ ps, const LeanRow<W> &r, int s,
                                         int S, int jstep, int k, bool last, unsigned o, unsigned xo, unsigned oj,
                                         unsigned oi, bool taps, Vec<W> &hxm, Vec<W> &hym) {
     const long long vol = p.vol;
@@ -480,7 +480,7 @@ __device__ __forceinline__ void e_tile(const StepParams<float> &p, const int jst
     const float *__restrict__ ring = p.ering + (long long)s * p.ering_stride;
     const float *__restrict__ Eo = ring + (long long)sl * 3 * p.vol;
     float *__restrict__ En = const_cast<float *>(ring) + (long long)slot_after(p, sl) * 3 * p.vol;
-    const float *__restrict__ H = p.H + (long long)s * 3 * vol;
+    const float *H = p.H + (long long)s * 3 * vol;
     float *__restrict__ ps = p.psiL + (long long)s * 12 * vol + 6 * vol;
     LeanRow<W> r;
     lean_row<W>(p, p.lx, p.ly, false, i, j, r);
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepPa
     const float *__restrict__ ring = p.ering + (long long)s * p.ering_stride;
     const float *__restrict__ Eo = ring + (long long)sl * 3 * p.vol;
     float *__restrict__ En = const_cast<float *>(ring) + (long long)slot_after(p, sl) * 3 * p.vol;
-    const float *__restrict__ H = p.H + (long long)s * 3 * vol;
+    const float *H = p.H + (long long)s * 3 * vol;        // plain loads: see pdl_wait
     float *__restrict__ ps = p.psiL + (long long)s * 12 * vol + 6 * vol;
     const int j0 = blockIdx.y * kLeanRows;
     const bool yblk = (j0 < npml) || (j0 + kLeanRows - 1 > p.ny - npml);
