@@ -660,7 +660,7 @@ __global__ void k_tap_inc(const StepParams<float> p, const int S, const int nste
         const double *T = p.T + (long long)n * p.J;
         double amp = 0.0;
         for (int jj = 0; jj < p.J; ++jj) amp += cf[jj] * T[jj];
-        const int o = tp.comp * (int)p.vol + (int)tp.idx;
+        const long long o = (long long)tp.comp * p.vol + tp.idx;   // up to 3 * 2^30
         v = (float)(-(double)p.cE[o] * tp.w * amp);
     }
     p.inc[t] = v;

@@ -1,4 +1,4 @@
-"""What the sources of the step kernels have to keep: the E kernels start while the H kernel drains (programmatic
+"""What the sources of the step kernels have to keep.  The E kernels start while the H kernel drains (programmatic
 dependent launch), so they read H through plain pointers.  A __restrict__ pointer to constant values would let a
 compiler read it as read-only data, above the wait for the H kernel."""
 import os
@@ -31,3 +31,13 @@ def test_e_kernels_read_h_through_plain_pointers(unit, names):
     for name, text in found.items():
         assert re.search(r"\*\s*H[xyz]?\b", text), name
         assert not re.search(r"__restrict__\s+H[xyz]?\b", text), name
+
+
+@pytest.mark.parametrize("unit", ["kern_lean.cu", "kern_ho.cu"])
+def test_indices_across_components_have_64_bits(unit):
+    """These kernels run on components of up to 2^30 entries, so an index into three of them does not fit 32 bits."""
+    assert 2 * (2 ** 30 - 1) + (2 ** 30 - 1) > 2 ** 31 - 1
+    with open(os.path.join(SRC, unit)) as f:
+        text = f.read()
+    assert not re.search(r"\(int\)\s*(p\.vol|tp\.idx)", text)
+    assert not re.search(r"\bint vol\b", text)
