@@ -166,9 +166,10 @@ int csem_estimate_adjoint_basis(double dt, int nt, const double *freqs_host, int
  * allocator (a framework's caching pool, a fixed arena) and must not see
  * foreign allocations, or run on a path where an allocation's implicit
  * synchronisation or possible failure is not acceptable.  This entry point
- * calls no cudaMalloc, cudaFree or other allocating routine: its work
- * vectors live in one file-scope device array of 8 MiB that every device
- * which loads the library keeps until the process exits.
+ * calls no cudaMalloc, cudaFree or other allocating routine: its phasor
+ * table lives in one file-scope device array of 4 MiB (the CG vectors are in
+ * shared memory), which every device that loads the library keeps until the
+ * process exits.
  *  Limits: nt <= 32768 and n_freq <= 8, else INVALID_ARG with a message.
  *  Every call looks the array's device address up (cudaGetSymbolAddress)
  *  with the caller's device current.  With lazy module loading (the CUDA
@@ -303,11 +304,11 @@ int csem_last_run_steps(csem_ctx *ctx, void *stream, int *steps);
 int csem_set_early_stop_volumes(csem_ctx *ctx, double tol, double floor_frac);
 
 /* Picks the launch shape of the H and E stepping kernels -- z planes per
- * thread (1, 2, 4, 8), the register budget (4, 6 or 8 resident 256-thread
- * blocks per SM), and for FP32 one or four cells per thread along x, the
- * bulk-copy-staged kernels (1, 2 or 4 rows per block, 2-16 planes) or the
- * lean four-cell kernels (1, 2 or 4 planes; see csem_set_launch) -- by
- * timing each candidate on n_src sources of this grid;
+ * thread (1, 2, 4, 8), the register budget (4, 6 or 8 resident blocks per SM,
+ * of 256 threads, or of 128 in the FP64 and lean kernels), and for FP32 one
+ * or four cells per thread along x, the bulk-copy-staged kernels (1, 2 or 4
+ * rows per block, 2-16 planes) or the lean one- and two-cell kernels (1, 2 or
+ * 4 planes; see csem_set_launch) -- by timing each candidate on n_src sources of this grid;
  * later calls use the fastest.  It then times the fused H+E step kernels (the
  * tiled one with z blocking 4, 8 or 16; for FP32 the one-pass, warp-specialised
  * and wave-ordered steps) against the best split pair and keeps the fastest, and

@@ -224,11 +224,14 @@ template <typename R>
 void axis_tab(const csem_ctx *c, int a, csem::AxisTab<R> &t) {
     const R *base = (const R *)c->d_tab;
     long long off = 0;
-    for (int b = 0; b < a; ++b) off += 9LL * (c->ax[b].n + 1);
+    for (int b = 0; b < a; ++b) off += (sizeof(R) == 8 ? 9LL : 6LL) * (c->ax[b].n + 1);
     const int n = c->ax[a].n;
-    t.c_h = base + off + 6 * (n + 1);
-    t.g_h = base + off + 7 * (n + 1);
-    t.g_n = base + off + 8 * (n + 1);
+    t.c_h = t.g_h = t.g_n = nullptr;
+    if (sizeof(R) == 8) {
+        t.c_h = base + off + 6 * (n + 1);
+        t.g_h = base + off + 7 * (n + 1);
+        t.g_n = base + off + 8 * (n + 1);
+    }
     t.ih_h = base + off;
     t.ih_n = base + off + (n + 1);
     t.b_h = base + off + 2 * (n + 1);
@@ -287,7 +290,6 @@ int upload_lean_tables(csem_ctx *c) {
         for (int i = 1; i < n; ++i) { v[4 * L + i] = (float)A.bn[i]; v[5 * L + i] = (float)A.an[i]; }
         tab.insert(tab.end(), v.begin(), v.end());
     }
-    tab.insert(tab.end(), 4, 0.f);   // zeros read by lanes off the x slab
     TRY(dalloc(c, &c->d_tabL, tab.size() * sizeof(float)));
     CK(cudaMemcpy(c->d_tabL, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice));
     return CSEM_OK;
@@ -325,13 +327,15 @@ int upload_tables(csem_ctx *c) {
         std::vector<R> ih_h(n + 1, R(0)), ih_n(n + 1, R(0)), bh(n + 1, R(0)), ah(n + 1, R(0)), bn(n + 1), an(n + 1);
         for (int i = 0; i < n; ++i) { ih_h[i] = (R)(1.0 / A.h[i]); bh[i] = (R)A.bh[i]; ah[i] = (R)A.ah[i]; }
         for (int i = 0; i <= n; ++i) { ih_n[i] = (R)(1.0 / A.ht[i]); bn[i] = (R)A.bn[i]; an[i] = (R)A.an[i]; }
-        std::vector<R> ch(n + 1, R(0)), gh(n + 1, R(0)), gn(n + 1);
+        for (auto *v : {&ih_h, &ih_n, &bh, &ah, &bn, &an}) tab.insert(tab.end(), v->begin(), v->end());
+        if (sizeof(R) != 8) continue;
+        std::vector<R> ch(n + 1, R(0)), gh(n + 1, R(0)), gn(n + 1);      // the FP64 kernels' tables
         for (int i = 0; i < n; ++i) {
             ch[i] = (R)(c->dt / kMu0 / A.h[i]);
             gh[i] = (R)(A.ah[i] * (c->dt / kMu0 / A.h[i]));
         }
         for (int i = 0; i <= n; ++i) gn[i] = (R)(A.an[i] / A.ht[i]);
-        for (auto *v : {&ih_h, &ih_n, &bh, &ah, &bn, &an, &ch, &gh, &gn}) tab.insert(tab.end(), v->begin(), v->end());
+        for (auto *v : {&ch, &gh, &gn}) tab.insert(tab.end(), v->begin(), v->end());
     }
     TRY(dalloc(c, (R **)&c->d_tab, tab.size() * sizeof(R)));
     CK(cudaMemcpy(c->d_tab, tab.data(), tab.size() * sizeof(R), cudaMemcpyHostToDevice));
@@ -474,7 +478,6 @@ csem::StepParams<R> step_params(csem_ctx *c, bool dft, void *acc) {
     p.LEAN_h = c->LEAN_h;
     p.LEAN_e = c->LEAN_e;
     p.lx = p.ly = p.lz = csem::AxisTab<R>{};
-    p.lzero = nullptr;
     p.FZ_by = 0; p.FZ_mb = 4; p.FZ_kz = 16; p.FZ_ws = 0;
     p.WAVE_lag = 0; p.WAVE_kz = 4; p.WAVE_mb = 8;
     p.wave = nullptr;
@@ -486,12 +489,7 @@ csem::StepParams<R> step_params(csem_ctx *c, bool dft, void *acc) {
     p.psiL = nullptr;
     p.cEm = nullptr;
     if constexpr (sizeof(R) == 4) {
-        if (c->d_tabL) {
-            lean_tab(c, 0, p.lx); lean_tab(c, 1, p.ly); lean_tab(c, 2, p.lz);
-            long long off = 0;
-            for (int a = 0; a < 3; ++a) off += 6LL * lean_len(c->ax[a].n);
-            p.lzero = (const float *)c->d_tabL + off;
-        }
+        if (c->d_tabL) { lean_tab(c, 0, p.lx); lean_tab(c, 1, p.ly); lean_tab(c, 2, p.lz); }
         p.psiL = c->d_psiL;
         p.cEm = c->d_cEm;
         p.wave = c->d_wave;
@@ -1971,7 +1969,7 @@ int csem_set_launch(csem_ctx *c, const int *cfg) {
     if (wv) {
         csem::StepParams<float> tp{};
         tp.nx = c->nx; tp.nz = c->nz; tp.psiL = c->d_psiL; tp.cEm = c->d_cEm; tp.wave = c->d_wave;
-        tp.lx.ih_n = c->d_tabL ? (const float *)c->d_tabL : nullptr; tp.lzero = tp.lx.ih_n;
+        tp.lx.ih_n = c->d_tabL ? (const float *)c->d_tabL : nullptr;
         if (c->precision != 32 || c->order != 2 || wv_lag < 1 || !csem::wave_supported(tp, wv_kz, wv_mb))
             return fail(CSEM_ERR_INVALID_ARG, "wave-ordered step: FP32, second order, nx a multiple of 4, lag >= 1, 2 or 4 planes, 6 or 8 blocks/SM");
     }

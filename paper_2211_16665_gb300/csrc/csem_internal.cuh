@@ -173,7 +173,6 @@ struct StepParams {
     int TMA_h, TMA_e;              // > 0: FP32 bulk-copy-staged kernels over this many rows per block
     int LEAN_h, LEAN_e;            // > 0: lean FP32 kernels with this many cells per thread (1 or 2)
     AxisTab<R> lx, ly, lz;         // the stepping tables padded to 16-byte groups (lean kernels)
-    const R *lzero;                // 4 zeros, 16-byte aligned (lean kernels)
     R *psiL;                       // [S][12][vol] CPML memory in the field layout (lean kernels)
     const R *cEm;                  // [3][vol] dt/eps, zero on the PEC edges (lean kernels)
     // fused one-pass FP32 step (kern_fz.cu): FZ_by rows per block (0: off), FZ_mb resident

@@ -723,7 +723,7 @@ bool lean_kz(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool
 
 cudaError_t launch_field_lean(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int w, int kz,
                               int mb) {
-    if (!p.psiL || !p.cEm || !p.lx.ih_n || !p.lzero) return cudaErrorInvalidValue;
+    if (!p.psiL || !p.cEm || !p.lx.ih_n) return cudaErrorInvalidValue;
     bool ok = false;
     if (w == 1 && mb == 6) ok = lean_kz<1, 6>(p, S, jstep, st, h, kz);
     else if (w == 1 && mb == 8) ok = lean_kz<1, 8>(p, S, jstep, st, h, kz);
@@ -736,7 +736,7 @@ cudaError_t launch_field_lean(const StepParams<float> &p, int S, int jstep, cuda
 }
 
 bool wave_supported(const StepParams<float> &p, int kz, int mb) {
-    return p.wave && p.nx % 4 == 0 && p.psiL && p.cEm && p.lx.ih_n && p.lzero && (kz == 2 || kz == 4) &&
+    return p.wave && p.nx % 4 == 0 && p.psiL && p.cEm && p.lx.ih_n && (kz == 2 || kz == 4) &&
            (mb == 6 || mb == 8) && p.nz <= kMaxWaveChunks * kz;
 }
 

@@ -21,14 +21,14 @@ namespace {
 
 constexpr int kNoAllocMaxNt = 32768;
 constexpr int kNoAllocMaxCols = 2 * csem::kMaxFreq;
-// layout: phasor table (at most half of [cols][2][nt]) | [cols][cols] Gram matrix | [1 + cols] scalars | [cols] int iteration counts
-constexpr size_t kVecDoubles = (size_t)kNoAllocMaxCols * 2 * kNoAllocMaxNt;
+// layout: phasor table ([cols][nt], nt rounded up) | [cols][cols] Gram matrix | [1 + cols] scalars | [cols] int iteration counts
+constexpr size_t kVecDoubles = (size_t)kNoAllocMaxCols * kNoAllocMaxNt;
 constexpr size_t kGramDoubles = (size_t)kNoAllocMaxCols * kNoAllocMaxCols;
 constexpr size_t kScalDoubles = 1 + kNoAllocMaxCols;
 constexpr size_t kIterDoubles = (kNoAllocMaxCols + 1) / 2;   // ints packed two per double
 constexpr size_t kScratchDoubles = kVecDoubles + kGramDoubles + kScalDoubles + kIterDoubles;
 
-__device__ __align__(256) double g_basis_scratch[kScratchDoubles];   // 8 MiB + a few KiB
+__device__ __align__(256) double g_basis_scratch[kScratchDoubles];   // 4 MiB + a few KiB
 
 // Host code cannot use g_basis_scratch's name as a device address.  Resolve it
 // on every call, with the caller's device current: once the module is loaded this
@@ -65,6 +65,8 @@ extern "C" int csem_estimate_adjoint_basis_noalloc(double dt, int nt, const doub
         }
         a[f] = std::sqrt(2.0 * M_PI * freqs[f] * 2.0 * M_PI * f0);
     }
+    if (csem::basis_scratch_doubles(nt, nf) > kVecDoubles)
+        return csem::set_last_error(CSEM_ERR_INVALID_ARG, "adjoint basis (no-alloc): sizes beyond its array");
     double *base = nullptr;
     int rc = scratch_for_current_device(&base);
     if (rc != CSEM_OK) return rc;
