@@ -126,6 +126,7 @@ int set_last_error(int code, const std::string &msg) { return fail(code, msg); }
 
 struct csem_ctx {
     int device = 0;
+    int sms = 152;                       // SMs of the device
     int nx, ny, nz, npml, NX, NY, NZ, pitch;
     long long plane, vol;
     Axis ax[3];
@@ -461,6 +462,7 @@ csem::StepParams<R> step_params(csem_ctx *c, bool dft, void *acc) {
     p.ering = (R *)c->d_ering;
     p.ering_stride = (long long)c->nslot * 3 * c->vol;
     p.nslot = c->nslot;
+    p.sms = c->sms;
     p.mslot = csem::slot_magic(c->nt, p.nslot);
     p.psi = (R *)c->d_psi;
     p.psi_stride = c->psi_stride; p.sx = c->sx; p.sy = c->sy; p.sz = c->sz;
@@ -1581,6 +1583,7 @@ int csem_create(csem_ctx **out, const csem_grid *g, const csem_opts *o) {
 
     csem_ctx *c = new csem_ctx();
     cudaGetDevice(&c->device);
+    if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) cudaGetLastError();
     c->nx = g->nx; c->ny = g->ny; c->nz = g->nz; c->npml = g->npml;
     c->NX = c->nx + 1; c->NY = c->ny + 1; c->NZ = c->nz + 1;
     c->pitch = (c->NX + 7) / 8 * 8;

@@ -65,16 +65,15 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t
 constexpr long long kFarBytes = 90LL << 20;
 inline bool far_fields(long long vol, int S) { return 12LL * vol * (3 * S + 1) > kFarBytes; }
 
-// z blocks of kz planes that fill whole waves of the GPU (`per` blocks to a z block, mb resident blocks per SM); the
+// z blocks of kz planes that fill whole waves of the GPU (`per` blocks to a z block, sms SMs with mb resident blocks each); the
 // planes after them go to blocks of one plane, which end the launch closer together.  With blocks of kz planes
 // throughout, the last wave left most of the GPU idle for the life of a block: 128 x 128 x 96 in 1536 blocks of four
 // planes is 1.3 waves.  Forward runs of 256 steps, without / with: 128 x 128 x 96 6.88 / 6.53 ms, 116^3 7.10 / 6.79,
 // 148 x 148 x 96 10.6 / 9.8, 188 x 188 x 96 14.8 / 14.3, four sources of 116^3 (5.5 waves) 29.1 / 28.4.  Launches of up
 // to 1.2 waves and of more than 8 stay as they are: one plane per block costs more than it gives there (72 x 68 x 60,
 // 1.1 waves: 5.15 / 5.35; two sources of 256 x 256 x 128, 13.5 waves: 68.3 / 68.5).
-constexpr int kSMs = 152;
-inline int big_blocks(int nzb, int kz, int per, int mb) {
-    const long long slots = (long long)kSMs * mb, total = (long long)nzb * per;
+inline int big_blocks(int sms, int nzb, int kz, int per, int mb) {
+    const long long slots = (long long)sms * mb, total = (long long)nzb * per;
     if (kz == 1 || 5 * total <= 6 * slots || total > 8 * slots) return nzb;
     return (int)(total / slots * slots / per);
 }
@@ -161,6 +160,7 @@ struct StepParams {
     R *ering;                      // [S][nslot][3][vol]
     long long ering_stride;        // nslot*3*vol
     int nslot;                     // transform block M + 1
+    int sms;                       // SMs of the device
     unsigned mslot;                // ceil(2^32 / nslot) where steps * nslot < 2^32, else 0 (see slot_of)
     R *psi;                        // [S][psi_stride]
     long long psi_stride, sx, sy, sz;

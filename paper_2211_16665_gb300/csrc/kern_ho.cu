@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(128, MINB) k_e_ho4(const StepParams<float> p, 
 template <int KZ, int MB>
 void go_ho4k(const StepParams<float> &p, const HoTab<float> &w, int S, int jstep, cudaStream_t st, bool h) {
     const int gx = (p.nx / 2 + 31) / 32, gy = (p.ny + 3) / 4, nzb = (p.nz + KZ - 1) / KZ;
-    const int nbig = big_blocks(nzb, KZ, gx * gy * S, MB);
+    const int nbig = big_blocks(p.sms, nzb, KZ, gx * gy * S, MB);
     const dim3 grid(gx, gy, (nbig + std::max(p.nz - nbig * KZ, 0)) * S);
     const unsigned mS = div_magic((unsigned)S);
     if (h) launch_pdl(k_h_ho4<KZ, MB>, grid, dim3(32, 4), st, p, w, jstep, (unsigned)S, mS, nbig);

@@ -700,7 +700,7 @@ template <int W, int KZ, int MB, bool F4>
 void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h) {
     const int nv = (p.nx + W - 1) / W, nzb = (p.nz + KZ - 1) / KZ;
     const int gx = (nv + kLeanX - 1) / kLeanX, gy = (p.ny + kLeanRows - 1) / kLeanRows;
-    const int nbig = big_blocks(nzb, KZ, gx * gy * S, MB);
+    const int nbig = big_blocks(p.sms, nzb, KZ, gx * gy * S, MB);
     if constexpr (KZ > 1)
         if (nbig < nzb) return lean_launch<W, KZ, MB, true, F4>(p, dim3(gx, gy, (nbig + p.nz - nbig * KZ) * S), nbig, S, jstep, st, h);
     lean_launch<W, KZ, MB, false, F4>(p, dim3(gx, gy, nzb * S), nzb, S, jstep, st, h);
