@@ -322,7 +322,11 @@ int csem_set_early_stop_volumes(csem_ctx *ctx, double tol, double floor_frac);
  * csem_set_launch), then the step's form: 0 split, 4/8/16 the fused z
  * blocking, 10000 + code the one-pass kernel, 30000 + code the
  * warp-specialised fused kernel, 50000 + code the wave-ordered step.  Overwrites the
- * context's field state and blocks until the timing is done.  In an FP32
+ * context's field state and blocks until the timing is done.  It also fixes how
+ * the second-order lean kernels round, by cells * n_src: the runs of a tuned
+ * context give the same bits whatever was picked (up to the flush's order of
+ * sums), and after csem_set_launch too.  In an untuned context the rounding
+ * follows the planes per thread.  In an FP32
  * second-order context whose nx is no multiple of 4 the first call allocates
  * the lean kernels' memory (12 volume arrays per source and three more) where
  * it fits in a quarter of the free memory.

@@ -127,6 +127,8 @@ int set_last_error(int code, const std::string &msg) { return fail(code, msg); }
 struct csem_ctx {
     int device = 0;
     int sms = 152;                       // SMs of the device
+    csem::Rounding rnd = {3, 3, 1, 0};   // of the lean kernels: set by csem_autotune, before it by csem_set_launch
+    bool tuned = false;
     int nx, ny, nz, npml, NX, NY, NZ, pitch;
     long long plane, vol;
     Axis ax[3];
@@ -463,6 +465,7 @@ csem::StepParams<R> step_params(csem_ctx *c, bool dft, void *acc) {
     p.ering_stride = (long long)c->nslot * 3 * c->vol;
     p.nslot = c->nslot;
     p.sms = c->sms;
+    p.rnd = c->rnd;
     p.mslot = csem::slot_magic(c->nt, p.nslot);
     p.psi = (R *)c->d_psi;
     p.psi_stride = c->psi_stride; p.sx = c->sx; p.sy = c->sy; p.sz = c->sz;
@@ -1342,6 +1345,8 @@ int time_impl(csem_ctx *c, int S, void *vol, int launches, double *ms, cudaStrea
 // Times the H and E kernels for every z-blocking candidate on S sources and keeps the fastest.
 template <typename R>
 int autotune_impl(csem_ctx *c, int S, cudaStream_t st) {
+    c->tuned = true;
+    c->rnd = csem::rounding_of((double)c->nx * c->ny * c->nz * S);
     // rows that are no multiple of four: only the autotuner brings the lean kernels there, so it takes their memory
     // (without it they are not among the candidates)
     if (sizeof(R) == 4 && c->order == 2 && !c->d_psiL && c->nx % 4 != 0 && lean_fits(c)) {
@@ -2032,6 +2037,7 @@ int csem_set_launch(csem_ctx *c, const int *cfg) {
     c->VEC_h = vh; c->VEC_e = ve;
     c->TMA_h = th; c->TMA_e = te;
     c->LEAN_h = lh; c->LEAN_e = le;
+    if (!c->tuned) c->rnd = csem::Rounding{(wv ? wv_kz : kzh) - 1, (wv ? wv_kz : kze) - 1, 1, 0};
     return CSEM_OK;
 }
 

@@ -149,6 +149,22 @@ struct GeoTab {            // per-axis FP32 widths for the fused one-pass step (
     const float *s;       // sum of the two primal widths next to a node [n+1] (2 x the dual width)
 };
 
+// Which products the lean second-order kernels fuse (kern_lean.cu).  Compiled from plain expressions, the lean kernels
+// fused by planes per thread, the four-cell and the scalar ones (which other rows than multiples of four ran) in two
+// more ways, so a result hung on the tuned configuration.  csem_autotune now fixes the choice by the size of a launch, as the
+// configurations that were picked there (0.03 to 17 million cells times sources, 70 grids of rows of four and 50 others,
+// each tuned twice): planes per thread in H 1 up to about 0.16 million, 2 up to 1.6, then 4; in E 1, 2 up to 11, then 4;
+// on other rows the scalar H kernel up to 0.2 million, then the four-cell one, and the scalar E kernel up to 1.8, then
+// the four-cell one.  A configuration pinned in an untuned context rounds as its planes per thread.
+struct Rounding {
+    int h_mask, e_mask;        // planes per thread - 1
+    int h_bf, e_bf;            // other rows: four-cell kernels (b psi fused; H: along x)
+};
+inline Rounding rounding_of(double cells) {
+    return Rounding{cells < 160e3 ? 0 : (cells < 1.6e6 ? 1 : 3), cells < 160e3 ? 0 : (cells < 11e6 ? 1 : 3),
+                    cells < 200e3 ? 0 : 1, cells < 1.8e6 ? 0 : 1};
+}
+
 template <typename R>
 struct StepParams {
     int nx, ny, nz, NX, NY, NZ, pitch, npml;
@@ -161,6 +177,7 @@ struct StepParams {
     long long ering_stride;        // nslot*3*vol
     int nslot;                     // transform block M + 1
     int sms;                       // SMs of the device
+    Rounding rnd;
     unsigned mslot;                // ceil(2^32 / nslot) where steps * nslot < 2^32, else 0 (see slot_of)
     R *psi;                        // [S][psi_stride]
     long long psi_stride, sx, sy, sz;

@@ -37,11 +37,18 @@
 // E^n past L1), and the launches themselves below about 10^5 cells.
 #include "csem_internal.cuh"
 
+// 0: everything but the instances for other rows than multiples of four; 1, 2: the H and the E instances for those
+#ifndef CSEM_LEAN_UNIT
+#define CSEM_LEAN_UNIT 0
+#endif
+
 namespace csem {
 
 namespace {
 
 constexpr int kLeanX = 32, kLeanRows = 4;
+// rows of a multiple of four cells, and others with the roundings of the scalar or of the four-cell kernels (Rounding)
+constexpr int kRowsFour = 0, kRowsScalar = 1, kRowsVec = 2;
 
 template <int W> struct Vec { float v[W]; };
 template <int W> __device__ __forceinline__ Vec<W> ldc(const float *p) {
@@ -100,10 +107,10 @@ template <int W> __device__ __forceinline__ Vec<W> zv() {
 }
 // The roundings are spelled out.  Left to itself the compiler fuses one product or the other of a sum of two, by
 // instance; a gradient multiplies such a difference by up to 10^4 (the adjoint basis is ill-conditioned), so it then
-// changes with every new instance of a kernel.  Here every instance with the same planes per thread gives the same
-// bits, whatever its cells per thread, blocks per SM, order and size of its z blocks.  Which products are fused follows
-// the kernels that were compiled from the plain expressions, so results are what they were: h_plane and e_plane say
-// where.
+// changes with every new instance of a kernel.  Here every instance gives the same bits, whatever its cells and planes
+// per thread, blocks per SM, order and size of its z blocks.  Which products are fused follows the kernels that were
+// compiled from the plain expressions, so results are what they were: h_plane and e_plane say where, and Rounding
+// (csem_internal.cuh) which of those kernels.
 // a - b
 template <int W> __device__ __forceinline__ Vec<W> dif(const Vec<W> &a, const Vec<W> &b) {
     Vec<W> r;
@@ -143,25 +150,28 @@ template <int W> __device__ __forceinline__ Vec<W> neg(const Vec<W> &a) {
     for (int e = 0; e < W; ++e) r.v[e] = -a.v[e];
     return r;
 }
-// CPML recursion psi <- b psi + a d, then d += psi (shared or per-cell b, a).  BF: b psi is fused to the rounded a d,
+// CPML recursion psi <- b psi + a d, then d += psi (shared or per-cell b, a).  bf: b psi is fused to the rounded a d,
 // else a d to the rounded b psi.
-template <bool BF> __device__ __forceinline__ void cpml1(float &ps, float &d, float b, float a) {
-    ps = BF ? fmaf(b, ps, __fmul_rn(a, d)) : fmaf(a, d, __fmul_rn(b, ps));
+__device__ __forceinline__ void cpml1(bool bf, float &ps, float &d, float b, float a) {
+    ps = bf ? fmaf(b, ps, __fmul_rn(a, d)) : fmaf(a, d, __fmul_rn(b, ps));
     d = __fadd_rn(d, ps);
 }
-template <int W, bool BF> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, float b, float a) {
+template <int W> __device__ __forceinline__ void cpml(bool bf, Vec<W> &ps, Vec<W> &d, float b, float a) {
 #pragma unroll
-    for (int e = 0; e < W; ++e) cpml1<BF>(ps.v[e], d.v[e], b, a);
+    for (int e = 0; e < W; ++e) cpml1(bf, ps.v[e], d.v[e], b, a);
 }
-template <int W, bool BF> __device__ __forceinline__ void cpml(Vec<W> &ps, Vec<W> &d, const Vec<W> &b, const Vec<W> &a) {
+template <int W> __device__ __forceinline__ void cpml(bool bf, Vec<W> &ps, Vec<W> &d, const Vec<W> &b, const Vec<W> &a) {
 #pragma unroll
-    for (int e = 0; e < W; ++e) cpml1<BF>(ps.v[e], d.v[e], b.v[e], a.v[e]);
+    for (int e = 0; e < W; ++e) cpml1(bf, ps.v[e], d.v[e], b.v[e], a.v[e]);
 }
-// u s - v and v - u s, the product rounded first or (fuse) fused to v
-template <int W> __device__ __forceinline__ Vec<W> mulsub(bool fuse, const Vec<W> &u, float s, const Vec<W> &v) {
+// u s - v and v - u s, the product rounded first or (fuse) fused to v.  RT: fuse is known at run time only; u times one
+// and then s fused, or u times s and then one fused, costs one multiplication where a select costs three instructions.
+template <int W, bool RT> __device__ __forceinline__ Vec<W> mulsub(bool fuse, const Vec<W> &u, float s, const Vec<W> &v) {
+    if constexpr (RT) return mad<W>(mul<W>(u, fuse ? 1.f : s), fuse ? s : 1.f, neg<W>(v));
     return fuse ? mad<W>(u, s, neg<W>(v)) : dif<W>(mul<W>(u, s), v);
 }
-template <int W> __device__ __forceinline__ Vec<W> submul(bool fuse, const Vec<W> &v, const Vec<W> &u, float s) {
+template <int W, bool RT> __device__ __forceinline__ Vec<W> submul(bool fuse, const Vec<W> &v, const Vec<W> &u, float s) {
+    if constexpr (RT) return mad<W>(mul<W>(u, fuse ? 1.f : s), fuse ? -s : -1.f, v);
     return fuse ? mad<W>(u, -s, v) : dif<W>(v, mul<W>(u, s));
 }
 // the W cells shifted by one: (prev, a0, .., a_{W-2}) and (a1, .., a_{W-1}, next)
@@ -211,34 +221,34 @@ __device__ __forceinline__ void lean_row(const StepParams<float> &p, const AxisT
 // Source term E^{n+1} -= dt/eps J'^{n+1/2} for the taps in plane k of one
 // column (first tap, count in cm): the increments were computed for the chunk's
 // steps by k_tap_inc, so each tap costs two independent loads.
-__device__ __forceinline__ float3 lean_taps(const int *__restrict__ tk, const float *__restrict__ inc, int k, int2 cm) {
-    float3 r = make_float3(0.f, 0.f, 0.f);
+__device__ __forceinline__ void lean_taps(const int *__restrict__ tk, const float *__restrict__ inc, int k, int2 cm,
+                                          float &x, float &y, float &z) {
     for (int u = cm.x; u < cm.x + cm.y; ++u) {
         const int code = __ldg(tk + u);
         const float v = __ldg(inc + u);
         if ((code >> 2) != k) continue;
-        if ((code & 3) == 0) r.x += v;
-        else if ((code & 3) == 1) r.y += v;
-        else r.z += v;
+        if ((code & 3) == 0) x += v;
+        else if ((code & 3) == 1) y += v;
+        else z += v;
     }
-    return r;
 }
 
 }  // namespace
 
 // One plane k of the H update for the thread's W cells; YZ: the y/z recursion
-// may apply (a block on a y or z slab); FAR: see kFarBytes.  F4: the row length is a multiple of four; there the
-// products of a difference off the slabs are fused, but for those of Hy and Hz in the last plane of a z block of KZ
-// planes (last), and b psi is fused in the recursions.  Other rows ran the four-cell H and the scalar E kernel before
-// the lean ones took them, and keep the roundings of those: no fused product off the slabs, in H b psi fused along x
-// and a d along y and z, in E a d.  o: byte offset of the cells in a component, xo: of their x-slab entries.  exc, eyc: Ex, Ey of plane k (in), of plane k+1 (out).
-template <int W, bool YZ, bool FAR, bool F4>
+// may apply (a block on a y or z slab); FAR: see kFarBytes.  ROWS: on rows of four the
+// products of a difference off the slabs are fused, but for those of Hy and Hz in the last of every group of planes
+// (last; GEN: known at run time only), and b psi is fused in the recursions.  On other rows no product is fused off the
+// slabs, and in the recursions a d, but along x b psi with the four-cell kernels' rounding.  o: byte offset of the cells in a component, xo: of their
+// x-slab entries.  exc, eyc: Ex, Ey of plane k (in), of plane k+1 (out).
+template <int W, bool YZ, bool FAR, bool GEN, int ROWS>
 __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float *__restrict__ E, float *__restrict__ H,
                                         float *__restrict__ ps, const LeanRow<W> &r, int k, bool last, unsigned o, unsigned xo,
                                         Vec<W> &exc, Vec<W> &eyc) {
     const long long vol = p.vol;
     const unsigned plane = 4u * (unsigned)p.plane, pitch = 4u * (unsigned)p.pitch;
     const int npml = p.npml;
+    constexpr bool four = ROWS == kRowsFour, bf = ROWS != kRowsScalar;
     const float *Ey = E + vol, *Ez = E + 2 * vol;
     float *Hy = H + vol, *Hz = H + 2 * vol;
     const Vec<W> ezc = ldc<W>(Ez, o);
@@ -266,31 +276,31 @@ __device__ __forceinline__ void h_plane(const StepParams<float> &p, const float 
     Vec<W> zy = dif<W>(ezj, ezc), yz = dif<W>(eyk, eyc), c;
     if constexpr (YZ) {
         zy = mul<W>(zy, r.ihy); yz = mul<W>(yz, ihz);
-        if (ys) { cpml<W, F4>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
-        if (zs) { cpml<W, F4>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
+        if (ys) { cpml<W>(four, q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
+        if (zs) { cpml<W>(four, q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
         c = dif<W>(zy, yz);
-    } else c = mulsub<W>(F4, zy, r.ihy, mul<W>(yz, ihz));
+    } else c = mulsub<W, false>(four, zy, r.ihy, mul<W>(yz, ihz));
     hx = mad<W>(c, -p.cH, hx);
     // Hy at (i+1/2, j, k+1/2)
     Vec<W> xz = dif<W>(exk, exc), zx = mul<W>(dif<W>(ezx, ezc), r.ihx);
     if constexpr (YZ) {
         xz = mul<W>(xz, ihz);
-        if (zs) { cpml<W, F4>(q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
+        if (zs) { cpml<W>(four, q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
     }
-    cpml<W, true>(q3, zx, r.bx, r.ax);
+    cpml<W>(bf, q3, zx, r.bx, r.ax);
     if (r.xs) stv<W>(px3, xo, q3);
     if constexpr (YZ) c = dif<W>(xz, zx);
-    else c = mulsub<W>(F4 && !last, xz, ihz, zx);
+    else c = mulsub<W, GEN && four>(four && !last, xz, ihz, zx);
     hy = mad<W>(c, -p.cH, hy);
     // Hz at (i+1/2, j+1/2, k)
     Vec<W> yx = mul<W>(dif<W>(eyx, eyc), r.ihx), xy = dif<W>(exj, exc);
-    cpml<W, true>(q4, yx, r.bx, r.ax);
+    cpml<W>(bf, q4, yx, r.bx, r.ax);
     if (r.xs) stv<W>(px4, xo, q4);
     if constexpr (YZ) {
         xy = mul<W>(xy, r.ihy);
-        if (ys) { cpml<W, F4>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
+        if (ys) { cpml<W>(four, q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
         c = dif<W>(yx, xy);
-    } else c = submul<W>(F4 && !last, yx, xy, r.ihy);
+    } else c = submul<W, GEN && four>(four && !last, yx, xy, r.ihy);
     hz = mad<W>(c, -p.cH, hz);
 
     if constexpr (FAR) { stl<W>(H, o, hx); stl<W>(Hy, o, hy); stl<W>(Hz, o, hz); }
@@ -327,19 +337,21 @@ __device__ __forceinline__ void h_tile(const StepParams<float> &p, const int jst
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, false, true>(p, E, H, ps, r, k, kk == KZ - 1, o, xo, exc, eyc);
-        else h_plane<W, false, false, true>(p, E, H, ps, r, k, kk == KZ - 1, o, xo, exc, eyc);
+        const bool last = (k & p.rnd.h_mask) == p.rnd.h_mask;
+        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, false, true, kRowsFour>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
+        else h_plane<W, false, false, true, kRowsFour>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
     }
 }
 
-template <int W, int KZ, int MINB, bool FAR, bool TAIL, bool F4>
+// GEN: the last z blocks have one plane (big_blocks), or groups of planes that round alike are not the z blocks.
+template <int W, int KZ, int MINB, bool FAR, bool GEN, int ROWS>
 __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepParams<float> p, const int jstep, const unsigned S,
                                                                        const unsigned mS, const int nbig) {
     const int i = (blockIdx.x * kLeanX + threadIdx.x) * W;
     const int j = blockIdx.y * kLeanRows + threadIdx.y;
     const int zb = (int)div_by(blockIdx.z, mS);   // the source runs fastest: the sources of one
     const int s = (int)(blockIdx.z - zb * S);     // z block follow one another
-    const bool one = TAIL && zb >= nbig;          // big_blocks
+    const bool one = GEN && zb >= nbig;           // big_blocks
     const int k0 = one ? nbig * KZ + (zb - nbig) : zb * KZ, k1 = min(k0 + (one ? 1 : KZ), p.nz);
     if (i >= p.nx || j >= p.ny) return;
     const int plane = (int)p.plane, npml = p.npml;
@@ -361,9 +373,9 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_h_lean(const StepPa
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        const bool last = TAIL ? (k & (KZ - 1)) == KZ - 1 : kk == KZ - 1;   // without big_blocks z blocks start at multiples of KZ
-        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, FAR, F4>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
-        else h_plane<W, false, FAR, F4>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
+        const bool last = GEN ? (k & p.rnd.h_mask) == p.rnd.h_mask : kk == KZ - 1;
+        if (yblk || k < npml || k >= p.nz - npml) h_plane<W, true, FAR, GEN, ROWS>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
+        else h_plane<W, false, FAR, GEN, ROWS>(p, E, H, ps, r, k, last, o, xo, exc, eyc);
     }
 }
 
@@ -383,15 +395,16 @@ template <bool CG> __device__ __forceinline__ float ldh1(const float *b, unsigne
 }
 
 // One plane k of the E update; o, xo as in h_plane; oj, oi: from o to the lower neighbours along y and x (0 on
-// the outer faces).  F4: off the slabs Ey's products are never fused, Ez's not in the last plane.  hxm, hym: Hx, Hy of
-// plane k-1 (in), of plane k (out).
-template <int W, bool YZ, bool CG, bool F4>
+// the outer faces).  ROWS, GEN: as in h_plane, but on rows of four Ey's products are never fused, and on
+// other rows all recursions fuse b psi with the four-cell kernels' rounding; hxm, hym: Hx, Hy of plane k-1 (in), of plane k (out).
+template <int W, bool YZ, bool CG, bool GEN, int ROWS>
 __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float *__restrict__ Eo, float *__restrict__ En,
                                         const float *H, float *__restrict__ ps, const LeanRow<W> &r, int s,
                                         int S, int jstep, int k, bool last, unsigned o, unsigned xo, unsigned oj,
                                         unsigned oi, bool taps, Vec<W> &hxm, Vec<W> &hym) {
     const long long vol = p.vol;
     const int npml = p.npml;
+    constexpr bool four = ROWS == kRowsFour, bf = ROWS != kRowsScalar;
     const float *__restrict__ cE = p.cEm;
     const float *Hy = H + vol, *Hz = H + 2 * vol;
     const Vec<W> hxc = ldh<W, CG>(H, o), hyc = ldh<W, CG>(Hy, o), hzc = ldh<W, CG>(Hz, o);
@@ -419,31 +432,31 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
     Vec<W> zy = dif<W>(hzc, hzj), yz = dif<W>(hyc, hym), c;
     if constexpr (YZ) {
         zy = mul<W>(zy, r.ihy); yz = mul<W>(yz, ihz);
-        if (ys) { cpml<W, F4>(q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
-        if (zs) { cpml<W, F4>(q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
+        if (ys) { cpml<W>(bf, q0, zy, r.by, r.ay); stv<W>(ps, o, q0); }
+        if (zs) { cpml<W>(bf, q1, yz, bz, az); stv<W>(ps + vol, o, q1); }
         c = dif<W>(zy, yz);
-    } else c = mulsub<W>(F4, zy, r.ihy, mul<W>(yz, ihz));
+    } else c = mulsub<W, false>(four, zy, r.ihy, mul<W>(yz, ihz));
     Vec<W> e0 = mad<W>(c, c0, eo0);
     // Ey at (i, j+1/2, k)
     Vec<W> xz = dif<W>(hxc, hxm), zx = mul<W>(dif<W>(hzc, hzx), r.ihx);
     if constexpr (YZ) {
         xz = mul<W>(xz, ihz);
-        if (zs) { cpml<W, F4>(q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
+        if (zs) { cpml<W>(bf, q2, xz, bz, az); stv<W>(ps + 2 * vol, o, q2); }
     }
-    cpml<W, F4>(q3, zx, r.bx, r.ax);
+    cpml<W>(bf, q3, zx, r.bx, r.ax);
     if (r.xs) stv<W>(px3, xo, q3);
     if constexpr (YZ) c = dif<W>(xz, zx);
-    else c = mulsub<W>(false, xz, ihz, zx);
+    else c = mulsub<W, false>(false, xz, ihz, zx);
     Vec<W> e1 = mad<W>(c, c1, eo1);
     // Ez at (i, j, k+1/2)
     Vec<W> yx = mul<W>(dif<W>(hyc, hyx), r.ihx), xy = dif<W>(hxc, hxj);
-    cpml<W, F4>(q4, yx, r.bx, r.ax);
+    cpml<W>(bf, q4, yx, r.bx, r.ax);
     if (r.xs) stv<W>(px4, xo, q4);
     if constexpr (YZ) {
         xy = mul<W>(xy, r.ihy);
-        if (ys) { cpml<W, F4>(q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
+        if (ys) { cpml<W>(bf, q5, xy, r.by, r.ay); stv<W>(ps + 5 * vol, o, q5); }
         c = dif<W>(yx, xy);
-    } else c = submul<W>(F4 && !last, yx, xy, r.ihy);
+    } else c = submul<W, GEN && four>(four && !last, yx, xy, r.ihy);
     Vec<W> e2 = mad<W>(c, c2, eo2);
 
     if (taps) {
@@ -453,7 +466,8 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
         for (int e = 0; e < W; ++e) {
             const int2 c = __ldg(cm + e);
             if (c.y == 0) continue;
-            const float3 a = lean_taps(tk, inc, k, c);
+            float3 a = make_float3(0.f, 0.f, 0.f);
+            lean_taps(tk, inc, k, c, a.x, a.y, a.z);
             e0.v[e] += a.x; e1.v[e] += a.y; e2.v[e] += a.z;
         }
     }
@@ -496,13 +510,14 @@ __device__ __forceinline__ void e_tile(const StepParams<float> &p, const int jst
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
+        const bool last = (k & p.rnd.e_mask) == p.rnd.e_mask;
         if (yblk || k < npml || k > p.nz - npml)
-            e_plane<W, true, CG, true>(p, Eo, En, H, ps, r, s, S, jstep, k, kk == KZ - 1, o, xo, oj, oi, taps, hxm, hym);
-        else e_plane<W, false, CG, true>(p, Eo, En, H, ps, r, s, S, jstep, k, kk == KZ - 1, o, xo, oj, oi, taps, hxm, hym);
+            e_plane<W, true, CG, true, kRowsFour>(p, Eo, En, H, ps, r, s, S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
+        else e_plane<W, false, CG, true, kRowsFour>(p, Eo, En, H, ps, r, s, S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
     }
 }
 
-template <int W, int KZ, int MINB, bool FAR, bool TAIL, bool F4>
+template <int W, int KZ, int MINB, bool FAR, bool GEN, int ROWS>
 __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepParams<float> p, const int jstep, const unsigned S,
                                                                        const unsigned mS, const int nbig) {
     const int i = (blockIdx.x * kLeanX + threadIdx.x) * W;
@@ -510,7 +525,7 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepPa
     const int zq = (int)div_by(blockIdx.z, mS);   // the source runs fastest: the sources of one z
     const int s = (int)(blockIdx.z - zq * S);     // block share the dt/eps reads in L2
     int k0 = (FAR ? (p.nz + KZ - 1) / KZ - 1 - zq : zq) * KZ, k1 = min(k0 + KZ, p.nz);   // downwards where FAR (kFarBytes)
-    if constexpr (TAIL) {                         // big_blocks
+    if constexpr (GEN) {                          // big_blocks
         const int at = zq < nbig ? zq * KZ : nbig * KZ + (zq - nbig), len = zq < nbig ? KZ : 1;
         k0 = FAR ? max(p.nz - at - len, 0) : at;
         k1 = FAR ? p.nz - at : min(at + len, p.nz);
@@ -539,11 +554,70 @@ __global__ void __launch_bounds__(kLeanX *kLeanRows, MINB) k_e_lean(const StepPa
     for (int kk = 0; kk < KZ; ++kk, o += 4u * (unsigned)plane, xo += dx) {
         const int k = k0 + kk;
         if (k >= k1) break;
-        const bool last = TAIL ? (k & (KZ - 1)) == KZ - 1 : kk == KZ - 1;   // without big_blocks z blocks start at multiples of KZ
-        if (yblk || k < npml || k > p.nz - npml) e_plane<W, true, false, F4>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
-        else e_plane<W, false, false, F4>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
+        const bool last = GEN ? (k & p.rnd.e_mask) == p.rnd.e_mask : kk == KZ - 1;
+        if (yblk || k < npml || k > p.nz - npml) e_plane<W, true, false, GEN, ROWS>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
+        else e_plane<W, false, false, GEN, ROWS>(p, Eo, En, H, ps, r, s, (int)S, jstep, k, last, o, xo, oj, oi, taps, hxm, hym);
     }
 }
+
+// Launches of one half (H or E) on rows of one kind; the kinds and halves are compiled in three units (see the end).
+namespace {
+template <int W, int KZ, int MB, int ROWS, bool H, bool GEN, bool FAR>
+void lean_launch(const StepParams<float> &p, dim3 grid, int nbig, int S, int jstep, cudaStream_t st) {
+    const dim3 block(kLeanX, kLeanRows);
+    const unsigned mS = div_magic((unsigned)S);
+    if constexpr (H) launch_pdl(k_h_lean<W, KZ, MB, FAR, GEN, ROWS>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+    else launch_pdl(k_e_lean<W, KZ, MB, FAR, GEN, ROWS>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
+}
+template <int ROWS, bool H, int W, int KZ, int MB>
+void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st) {
+    const int nv = (p.nx + W - 1) / W, nzb = (p.nz + KZ - 1) / KZ;
+    const int gx = (nv + kLeanX - 1) / kLeanX, gy = (p.ny + kLeanRows - 1) / kLeanRows;
+    const int nbig = big_blocks(p.sms, nzb, KZ, gx * gy * S, MB);
+    const dim3 grid(gx, gy, (nbig < nzb ? nbig + p.nz - nbig * KZ : nzb) * S);
+    const bool gen = nbig < nzb || (ROWS == kRowsFour && (H ? p.rnd.h_mask : p.rnd.e_mask) != KZ - 1);
+    const bool far = far_fields(p.vol, S);
+    if constexpr (KZ > 1 || ROWS == kRowsFour) {
+        if (gen && far) return lean_launch<W, KZ, MB, ROWS, H, true, true>(p, grid, nbig, S, jstep, st);
+        if (gen) return lean_launch<W, KZ, MB, ROWS, H, true, false>(p, grid, nbig, S, jstep, st);
+    }
+    if (far) lean_launch<W, KZ, MB, ROWS, H, false, true>(p, grid, nbig, S, jstep, st);
+    else lean_launch<W, KZ, MB, ROWS, H, false, false>(p, grid, nbig, S, jstep, st);
+}
+template <int ROWS, bool H, int W, int MB>
+bool lean_kz(const StepParams<float> &p, int S, int jstep, cudaStream_t st, int kz) {
+    switch (kz) {
+        case 1: lean_go<ROWS, H, W, 1, MB>(p, S, jstep, st); return true;
+        case 2: lean_go<ROWS, H, W, 2, MB>(p, S, jstep, st); return true;
+        case 4: lean_go<ROWS, H, W, 4, MB>(p, S, jstep, st); return true;
+        default: return false;
+    }
+}
+template <int ROWS, bool H>
+bool lean_half(const StepParams<float> &p, int S, int jstep, cudaStream_t st, int w, int kz, int mb) {
+    if (w == 1 && mb == 6) return lean_kz<ROWS, H, 1, 6>(p, S, jstep, st, kz);
+    if (w == 1 && mb == 8) return lean_kz<ROWS, H, 1, 8>(p, S, jstep, st, kz);
+    if (w == 2 && mb == 4) return lean_kz<ROWS, H, 2, 4>(p, S, jstep, st, kz);
+    if (w == 2 && mb == 6) return lean_kz<ROWS, H, 2, 6>(p, S, jstep, st, kz);
+    if (w == 2 && mb == 8) return lean_kz<ROWS, H, 2, 8>(p, S, jstep, st, kz);
+    return false;
+}
+}  // namespace
+
+// The instances for other rows than multiples of four: kern_lean_h.cu and kern_lean_e.cu.
+bool lean_other_h(const StepParams<float> &p, int S, int jstep, cudaStream_t st, int w, int kz, int mb);
+bool lean_other_e(const StepParams<float> &p, int S, int jstep, cudaStream_t st, int w, int kz, int mb);
+#if CSEM_LEAN_UNIT == 1
+bool lean_other_h(const StepParams<float> &p, int S, int jstep, cudaStream_t st, int w, int kz, int mb) {
+    return p.rnd.h_bf ? lean_half<kRowsVec, true>(p, S, jstep, st, w, kz, mb)
+                      : lean_half<kRowsScalar, true>(p, S, jstep, st, w, kz, mb);
+}
+#elif CSEM_LEAN_UNIT == 2
+bool lean_other_e(const StepParams<float> &p, int S, int jstep, cudaStream_t st, int w, int kz, int mb) {
+    return p.rnd.e_bf ? lean_half<kRowsVec, false>(p, S, jstep, st, w, kz, mb)
+                      : lean_half<kRowsScalar, false>(p, S, jstep, st, w, kz, mb);
+}
+#else
 
 // One whole step (H then E) in one launch, ordered by tickets: every block takes the next
 // ticket from a counter, and the tickets run through the z blocks ("chunks") as
@@ -685,51 +759,12 @@ __global__ void k_mask_coef(const StepParams<float> p, const float *__restrict__
     cEm[t] = ok ? cE[t] : 0.f;
 }
 
-namespace {
-template <int W, int KZ, int MB, bool TAIL, bool F4>
-void lean_launch(const StepParams<float> &p, dim3 grid, int nbig, int S, int jstep, cudaStream_t st, bool h) {
-    const dim3 block(kLeanX, kLeanRows);
-    const unsigned mS = div_magic((unsigned)S);
-    const bool far = far_fields(p.vol, S);
-    if (h && far) launch_pdl(k_h_lean<W, KZ, MB, true, TAIL, F4>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
-    else if (h) launch_pdl(k_h_lean<W, KZ, MB, false, TAIL, F4>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
-    else if (far) launch_pdl(k_e_lean<W, KZ, MB, true, TAIL, F4>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
-    else launch_pdl(k_e_lean<W, KZ, MB, false, TAIL, F4>, grid, block, st, p, jstep, (unsigned)S, mS, nbig);
-}
-template <int W, int KZ, int MB, bool F4>
-void lean_go(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h) {
-    const int nv = (p.nx + W - 1) / W, nzb = (p.nz + KZ - 1) / KZ;
-    const int gx = (nv + kLeanX - 1) / kLeanX, gy = (p.ny + kLeanRows - 1) / kLeanRows;
-    const int nbig = big_blocks(p.sms, nzb, KZ, gx * gy * S, MB);
-    if constexpr (KZ > 1)
-        if (nbig < nzb) return lean_launch<W, KZ, MB, true, F4>(p, dim3(gx, gy, (nbig + p.nz - nbig * KZ) * S), nbig, S, jstep, st, h);
-    lean_launch<W, KZ, MB, false, F4>(p, dim3(gx, gy, nzb * S), nzb, S, jstep, st, h);
-}
-template <int W, int KZ, int MB>
-void lean_rows(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h) {
-    if (p.nx % 4 == 0) lean_go<W, KZ, MB, true>(p, S, jstep, st, h);
-    else lean_go<W, KZ, MB, false>(p, S, jstep, st, h);
-}
-template <int W, int MB>
-bool lean_kz(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int kz) {
-    switch (kz) {
-        case 1: lean_rows<W, 1, MB>(p, S, jstep, st, h); return true;
-        case 2: lean_rows<W, 2, MB>(p, S, jstep, st, h); return true;
-        case 4: lean_rows<W, 4, MB>(p, S, jstep, st, h); return true;
-        default: return false;
-    }
-}
-}  // namespace
-
 cudaError_t launch_field_lean(const StepParams<float> &p, int S, int jstep, cudaStream_t st, bool h, int w, int kz,
                               int mb) {
     if (!p.psiL || !p.cEm || !p.lx.ih_n) return cudaErrorInvalidValue;
-    bool ok = false;
-    if (w == 1 && mb == 6) ok = lean_kz<1, 6>(p, S, jstep, st, h, kz);
-    else if (w == 1 && mb == 8) ok = lean_kz<1, 8>(p, S, jstep, st, h, kz);
-    else if (w == 2 && mb == 4) ok = lean_kz<2, 4>(p, S, jstep, st, h, kz);
-    else if (w == 2 && mb == 6) ok = lean_kz<2, 6>(p, S, jstep, st, h, kz);
-    else if (w == 2 && mb == 8) ok = lean_kz<2, 8>(p, S, jstep, st, h, kz);
+    bool ok;
+    if (p.nx % 4 != 0) ok = h ? lean_other_h(p, S, jstep, st, w, kz, mb) : lean_other_e(p, S, jstep, st, w, kz, mb);
+    else ok = h ? lean_half<kRowsFour, true>(p, S, jstep, st, w, kz, mb) : lean_half<kRowsFour, false>(p, S, jstep, st, w, kz, mb);
     if (!ok) return cudaErrorInvalidValue;
     g_launches++;
     return cudaGetLastError();
@@ -767,5 +802,7 @@ cudaError_t launch_mask_coef(const StepParams<float> &p, const float *cE, float 
     g_launches++;
     return cudaGetLastError();
 }
+
+#endif  // CSEM_LEAN_UNIT
 
 }  // namespace csem

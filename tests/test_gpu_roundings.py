@@ -1,6 +1,7 @@
 """Roundings of the FP32 step kernels.  Gradients multiply a rounding difference by up to 10^4 (the adjoint basis is
 ill-conditioned), so the kernels spell their roundings out: traces equal the stored ones of the same kernels compiled
-from plain expressions, and every instance with the same planes per thread gives the same bits."""
+from plain expressions, and every instance with the same planes per thread (in a tuned context: every instance) gives
+the same bits."""
 import json
 import os
 
@@ -58,6 +59,27 @@ def test_instances_give_the_same_bits(kz):
         assert torch.equal(d, out[0][0]) and torch.equal(E, out[0][1])
 
 
+# A tuned context fixes its rounding by the size of a launch: the same bits for every configuration, planes per thread
+# among them, and for every tuning
+@pytest.mark.parametrize("n,S", [(24, 1), (24, 3), (84, 1), (84, 3)])
+def test_tuned_contexts_give_the_same_bits(n, S):
+    from paper_2211_16665_gb300.engine import Engine
+    wl = W.small_box(n_core=n, n_core_y=n - 4, n_core_z=n - 3, npml=6, n_freq=2, nt=64, n_rec=4)
+    x, z = wl.src.x[0], wl.src.z[0]
+    src = W.Points.make([[x, 0.0, z], [x - 40.0, 90.0, z + 30.0], [x + 60.0, -50.0, z]][:S], [0, 1, 2][:S])
+    out = []
+    for again in range(2):
+        eng = Engine.from_workload(wl, max_src=S)
+        rho = eng.model_tensor(wl.rho_true)
+        for w, kz, mb in ((1, 1, 6), (2, 1, 8), (1, 2, 8), (2, 2, 4), (1, 4, 6), (2, 4, 8)):
+            eng.set_launch(kz_h=kz, mb_h=mb, lean_h=w, kz_e=kz, mb_e=mb, lean_e=w, block=16, flush_mode=0)
+            out.append(eng.fwd_model(rho, src, wl.rec, keep_volume=True))
+        eng.check()
+        eng.close()
+    for d, E in out[1:]:
+        assert torch.equal(d, out[0][0]) and torch.equal(E, out[0][1])
+
+
 # Fourth order: the same bits for every planes per thread and blocks per SM, with and without one-plane blocks
 @pytest.mark.parametrize("nx", [96, 82])
 def test_fourth_order_instances_give_the_same_bits(nx):
@@ -76,8 +98,8 @@ def test_fourth_order_instances_give_the_same_bits(nx):
         assert torch.equal(d, out[0][0]) and torch.equal(E, out[0][1])
 
 
-# Rows that are no multiple of four: the lean kernels round as the four-cell H and the scalar E kernel that ran there
-# before.  118 x 93 x 97 cells with three sources exceed L2 (E walks z downwards), with one some launches end in
+# Rows that are no multiple of four: the lean kernels round as the scalar or four-cell kernels that were picked there
+# before, by the size of a launch.  118 x 93 x 97 cells with three sources exceed L2 (E walks z downwards), with one some launches end in
 # one-plane blocks.
 @pytest.mark.parametrize("nx,ny,nz,npml,S", [(47, 39, 41, 8, 2), (42, 37, 38, 5, 1), (118, 93, 97, 7, 3),
                                              (111, 93, 97, 6, 1)])
@@ -92,7 +114,9 @@ def test_other_rows_round_as_the_general_kernels(nx, ny, nz, npml, S):
     rho = eng.model_tensor(wl.rho_true)
     out = []
     for w, kz, mb in ((0, 1, 4), (1, 1, 8), (1, 4, 6), (2, 1, 6), (2, 2, 4), (2, 2, 8), (2, 4, 6)):
-        eng.set_launch(kz_h=kz, mb_h=mb, lean_h=w, vec_h=int(w == 0), kz_e=kz, mb_e=mb, lean_e=w)
+        cells = nx * ny * nz * S
+        eng.set_launch(kz_h=kz, mb_h=mb, lean_h=w, vec_h=int(w == 0 and cells >= 200e3), kz_e=kz, mb_e=mb, lean_e=w,
+                       vec_e=int(w == 0 and cells >= 1.8e6))
         d, E = eng.fwd_model(rho, src, wl.rec, keep_volume=True)
         out.append((d, E))
     eng.check()
