@@ -396,7 +396,8 @@ template <bool CG> __device__ __forceinline__ float ldh1(const float *b, unsigne
 
 // One plane k of the E update; o, xo as in h_plane; oj, oi: from o to the lower neighbours along y and x (0 on
 // the outer faces).  ROWS, GEN: as in h_plane, but on rows of four Ey's products are never fused, and on
-// other rows all recursions fuse b psi with the four-cell kernels' rounding; hxm, hym: Hx, Hy of plane k-1 (in), of plane k (out).
+// other rows all recursions fuse b psi with the four-cell kernels' rounding; there the taps are added one by one, as the
+// general kernels add them.  hxm, hym: Hx, Hy of plane k-1 (in), of plane k (out).
 template <int W, bool YZ, bool CG, bool GEN, int ROWS>
 __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float *__restrict__ Eo, float *__restrict__ En,
                                         const float *H, float *__restrict__ ps, const LeanRow<W> &r, int s,
@@ -466,9 +467,11 @@ __device__ __forceinline__ void e_plane(const StepParams<float> &p, const float 
         for (int e = 0; e < W; ++e) {
             const int2 c = __ldg(cm + e);
             if (c.y == 0) continue;
-            float3 a = make_float3(0.f, 0.f, 0.f);
-            lean_taps(tk, inc, k, c, a.x, a.y, a.z);
-            e0.v[e] += a.x; e1.v[e] += a.y; e2.v[e] += a.z;
+            if constexpr (four) {
+                float3 a = make_float3(0.f, 0.f, 0.f);
+                lean_taps(tk, inc, k, c, a.x, a.y, a.z);
+                e0.v[e] += a.x; e1.v[e] += a.y; e2.v[e] += a.z;
+            } else lean_taps(tk, inc, k, c, e0.v[e], e1.v[e], e2.v[e]);
         }
     }
     stv<W>(En, o, e0);

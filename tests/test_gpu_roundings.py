@@ -99,7 +99,7 @@ def test_fourth_order_instances_give_the_same_bits(nx):
 
 
 # Rows that are no multiple of four: the lean kernels round as the scalar or four-cell kernels that were picked there
-# before, by the size of a launch.  118 x 93 x 97 cells with three sources exceed L2 (E walks z downwards), with one some launches end in
+# before, by the size of a launch, and add the taps of an edge one by one as they do.  118 x 93 x 97 cells with three sources exceed L2 (E walks z downwards), with one some launches end in
 # one-plane blocks.
 @pytest.mark.parametrize("nx,ny,nz,npml,S", [(47, 39, 41, 8, 2), (42, 37, 38, 5, 1), (118, 93, 97, 7, 3),
                                              (111, 93, 97, 6, 1)])
@@ -112,14 +112,18 @@ def test_other_rows_round_as_the_general_kernels(nx, ny, nz, npml, S):
     eng = Engine.from_workload(wl, max_src=S)
     assert eng.nx == nx
     rho = eng.model_tensor(wl.rho_true)
+    near = W.Points.make([[x + 9.0 * r, 5.0 * r, z] for r in range(5)], [0, 1, 0, 2, 0])   # they share edges
+    resid = torch.randn((S, near.n, 2), generator=torch.Generator().manual_seed(1), dtype=torch.complex128).to(rho.device)
+    basis, _, _ = eng.estimate_adjoint_basis()
     out = []
     for w, kz, mb in ((0, 1, 4), (1, 1, 8), (1, 4, 6), (2, 1, 6), (2, 2, 4), (2, 2, 8), (2, 4, 6)):
         cells = nx * ny * nz * S
         eng.set_launch(kz_h=kz, mb_h=mb, lean_h=w, vec_h=int(w == 0 and cells >= 200e3), kz_e=kz, mb_e=mb, lean_e=w,
                        vec_e=int(w == 0 and cells >= 1.8e6))
         d, E = eng.fwd_model(rho, src, wl.rec, keep_volume=True)
-        out.append((d, E))
+        V = eng.adjoint_model(rho, near, resid, basis)
+        out.append((d, E, V))
     eng.check()
     eng.close()
-    for d, E in out[1:]:
-        assert torch.equal(d, out[0][0]) and torch.equal(E, out[0][1])
+    for got in out[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(got, out[0]))
