@@ -634,7 +634,7 @@ cudaError_t launch_misfit(int n, const double *d_obs, const double *d_syn, const
 // keeps the column's CG vectors in shared memory (k_basis_cg).  Every sum is taken over the ranges
 // in the order of one block of kBT threads, so the results are those of that block.  Eight
 // frequencies, 19 492 steps, three solves of up to 200 iterations: 469 ms with one block per column
-// and phasors advanced in every pass, 38 ms now.
+// and phasors advanced in every pass, 43 ms now.
 // ---------------------------------------------------------------------------
 constexpr int kBT = 512;                 // ranges per column
 constexpr int kBC = 8;                   // SMs (CTAs of a cluster) per column

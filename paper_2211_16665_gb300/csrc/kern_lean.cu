@@ -13,9 +13,8 @@
 //  * the coefficient tables are padded to whole 16-byte groups, and the CPML
 //    coefficients are zero off the slabs and on the outer nodes.  A cell in the
 //    rounded-out slab but not in the CPML keeps psi = 0;
-//  * the x-slab recursion runs on every lane (lanes off the slab read zeros and
-//    have zero coefficients) and only slab lanes store, so warps do not diverge
-//    on it;
+//  * the x-slab recursion runs on every lane (lanes off the slab start from zero and
+//    have zero coefficients) and only slab lanes load and store;
 //  * a block whose plane is off the z slabs and whose rows are off the y slabs
 //    takes a code path without the y/z recursion, with fewer live values;
 //  * E is advanced with dt/eps set to zero on the PEC edges (tangential E on the
